@@ -4,7 +4,8 @@
 // that the same scores come out bit for bit on every run and agree with any
 // other implementation that follows the same written order):
 //   * feature slot k:  x = (float)((t(raw) - mu[k]) / sd[k]) with the slot
-//     transform t (identity, log1p, log) and the arithmetic in double;
+//     transform t (identity, log1p, log) and the arithmetic in double (here
+//     and below: canon_math.cuh computes the same rounded values without it);
 //   * every dot product starts from its bias (0 for the quality score) and
 //     accumulates acc = fma(w[k], x[k], acc) for k ascending, one rounding per
 //     step; the two query slots are the last two features, so the
@@ -22,6 +23,7 @@
 #include <cuda_bf16.h>
 #include <math.h>
 
+#include "canon_math.cuh"
 #include "hwr_internal.cuh"
 #include "select.cuh"
 #include "umma.cuh"
@@ -31,36 +33,19 @@ namespace hwr {
 // ---------------------------------------------------------------------------
 // scalar pieces
 
-__device__ __forceinline__ float standardise(uint8_t code, double raw, float mu,
-                                             float sd) {
-    double t = raw;
-    if (code == 1) t = log1p(raw);
-    else if (code == 2) t = log(raw);
-    return (float)((t - (double)mu) / (double)sd);
-}
-
-__device__ __forceinline__ float softplus_c(float z) {
-    double zd = (double)z;
-    return (float)(fmax(zd, 0.0) + log1p(exp(-fabs(zd))));
-}
-
-__device__ __forceinline__ float sigmoid_c(float s) {
-    return (float)(1.0 / (1.0 + exp(-(double)s)));
-}
-
 // Raw value of deployment feature slot k < F - 2 (layout in hwr.h).
-__device__ double deployment_raw(const Model &m, int d, int k, int32_t running) {
+__device__ ff deployment_raw(const Model &m, int d, int k, int32_t running) {
     const int M = m.M, P = m.P;
-    if (k < M) return m.dep_model[d] == k ? 1.0 : 0.0;
-    if (k < P) return m.dep_gpu[d] == k - M ? 1.0 : 0.0;
-    if (k == P) return (double)m.log10p[m.dep_model[d]];
-    if (k == P + 1) return (double)running;
-    if (k == P + 2) return (double)m.waiting[d];
-    if (k == P + 3) return (double)m.kv[d];
-    if (k == P + 4) return (double)m.gpu_util[d];
-    if (k == P + 5) return (double)m.ttft[d];
-    if (k == P + 6) return (double)m.tpot[d];
-    return 0.0;
+    if (k < M) return ff{m.dep_model[d] == k ? 1.f : 0.f, 0.f};
+    if (k < P) return ff{m.dep_gpu[d] == k - M ? 1.f : 0.f, 0.f};
+    if (k == P) return ff{m.log10p[m.dep_model[d]], 0.f};
+    if (k == P + 1) return ff_count(running);
+    if (k == P + 2) return ff_count(m.waiting[d]);
+    if (k == P + 3) return ff{m.kv[d], 0.f};
+    if (k == P + 4) return ff{m.gpu_util[d], 0.f};
+    if (k == P + 5) return ff{m.ttft[d], 0.f};
+    if (k == P + 6) return ff{m.tpot[d], 0.f};
+    return ff{0.f, 0.f};
 }
 
 __device__ __forceinline__ float emb_at(const void *emb, int bf16, size_t i) {
@@ -498,13 +483,13 @@ __global__ void __launch_bounds__(ROUTE_THREADS, CPT <= 4 ? 3 : 2) k_route_simt(
         // the two query slots on two warps (their fp64 chains run side by side)
         if (tid < QB) {
             const int qq = q0 + tid;
-            us[tid] = qq < q.Q ? standardise(m.xform[F - 2], (double)q.in_len[qq], m.mu[F - 2],
+            us[tid] = qq < q.Q ? standardise(m.xform[F - 2], q.in_len[qq], m.mu[F - 2],
                                              m.sd[F - 2])
                                : 0.f;
         } else if (tid >= 64 && tid < 64 + QB) {
             const int qi = tid - 64, qq = q0 + qi;
             const float o = qq < q.Q ? q.out_len[qq] : 0.f;
-            vs[qi] = qq < q.Q ? standardise(m.xform[F - 1], (double)o, m.mu[F - 1], m.sd[F - 1])
+            vs[qi] = qq < q.Q ? standardise(m.xform[F - 1], o, m.mu[F - 1], m.sd[F - 1])
                               : 0.f;
             ol[qi] = o;
         }
@@ -608,10 +593,10 @@ k_seq_prep(Model m, Queries q, int Qs, float *aux, uint16_t *pre_bf, int32_t *dm
     if ((int)blockIdx.x < nuv) {
         const int t = blockIdx.x * PREP_THREADS + tid;
         if (t < Qs) {
-            a.us[t] = standardise(m.xform[F - 2], (double)q.in_len[t], m.mu[F - 2], m.sd[F - 2]);
+            a.us[t] = standardise(m.xform[F - 2], q.in_len[t], m.mu[F - 2], m.sd[F - 2]);
         } else if (t < 2 * Qs) {
             const int i = t - Qs;
-            a.vs[i] = standardise(m.xform[F - 1], (double)q.out_len[i], m.mu[F - 1], m.sd[F - 1]);
+            a.vs[i] = standardise(m.xform[F - 1], q.out_len[i], m.mu[F - 1], m.sd[F - 1]);
         }
         return;
     }
@@ -622,7 +607,7 @@ k_seq_prep(Model m, Queries q, int Qs, float *aux, uint16_t *pre_bf, int32_t *dm
     const int g0 = d * (Qs + 1) + c0;
     __shared__ float xr[PREP_COUNTS];
     if (tid < cn) {
-        const float v = standardise(m.xform[P + 1], (double)(m.running[d] + c0 + tid), m.mu[P + 1],
+        const float v = standardise(m.xform[P + 1], ff_count(m.running[d] + c0 + tid), m.mu[P + 1],
                                     m.sd[P + 1]);
         xr[tid] = v;
         a.xr[g0 + tid] = v;
@@ -1201,10 +1186,10 @@ __device__ __forceinline__ void pair_cols_split(const Model &m, const Queries &q
     }
     // the query slots of the group's queries (fp64 chains side by side)
     if (tid < nq) {
-        qu[tid] = standardise(m.xform[F - 2], (double)q.in_len[q0 + tid], m.mu[F - 2], m.sd[F - 2]);
+        qu[tid] = standardise(m.xform[F - 2], q.in_len[q0 + tid], m.mu[F - 2], m.sd[F - 2]);
     } else if (tid >= 32 && tid < 32 + nq) {
         const float o = q.out_len[q0 + tid - 32];
-        qv[tid - 32] = standardise(m.xform[F - 1], (double)o, m.mu[F - 1], m.sd[F - 1]);
+        qv[tid - 32] = standardise(m.xform[F - 1], o, m.mu[F - 1], m.sd[F - 1]);
         qo[tid - 32] = o;
     }
     // this thread's unit k of layer 1 for every pair of the group: the
@@ -1390,9 +1375,9 @@ __device__ __forceinline__ void pair_cols_fused(const Model &m, const Queries &q
     }
     // the query slots of the group's queries (fp64 chains side by side)
     if (tid < nq) {
-        qu[tid] = standardise(m.xform[F - 2], (double)iv, m.mu[F - 2], m.sd[F - 2]);
+        qu[tid] = standardise(m.xform[F - 2], iv, m.mu[F - 2], m.sd[F - 2]);
     } else if (tid >= 32 && tid < 32 + nq) {
-        qv[tid - 32] = standardise(m.xform[F - 1], (double)ov, m.mu[F - 1], m.sd[F - 1]);
+        qv[tid - 32] = standardise(m.xform[F - 1], ov, m.mu[F - 1], m.sd[F - 1]);
         qo[tid - 32] = ov;
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
