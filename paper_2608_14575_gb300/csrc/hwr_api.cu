@@ -855,7 +855,7 @@ static hwr_status run_kernels(hwr_ctx *c, const Queries &q, uint32_t flags, bool
         CK(c, launch_route_pairs(m, q, c->pairC, c->pairQ, c->pairH, c->pairN, c->nsm, c->stream),
            "route kernel");
     else
-        CK(c, launch_route_simt(m, q, c->stream), "route kernel");
+        CK(c, launch_route_simt(m, q, c->nsm, c->status_d, c->stream), "route kernel");
     a.done();
     return HWR_OK;
 }
@@ -1182,8 +1182,7 @@ static hwr_status route_impl(hwr_ctx *c, int32_t Q, const float *in_len, const f
     c->async_pending = false;
     c->snap_busy = false;
     CK(c, cudaGetLastError(), "kernel");
-    if (tensor || (seq && (flags & HWR_PATH_TENSOR))) TRY(check_status_word(c));
-    return HWR_OK;
+    return check_status_word(c);
 }
 
 extern "C" hwr_status hwr_route_batch(hwr_ctx *c, int32_t Q, const float *in_len,

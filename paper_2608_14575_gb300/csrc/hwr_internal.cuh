@@ -114,8 +114,10 @@ __device__ __forceinline__ float query_budget(const Queries &q, int row) {
 // waiting, kv, gpu_util, ttft, tpot) into the six device arrays, which m.running
 // starts (they are contiguous, in that order).
 cudaError_t launch_snapshot(const Model &m, const uint32_t *stage, cudaStream_t s);
-// Fused gather -> MLP -> mask -> argmax for a batch.
-cudaError_t launch_route_simt(const Model &m, const Queries &q, cudaStream_t s);
+// Fused gather -> MLP -> mask -> argmax for a batch, on nsm SMs.  status: the
+// device status word (bounded waits).
+cudaError_t launch_route_simt(const Model &m, const Queries &q, int nsm, int32_t *status,
+                              cudaStream_t s);
 // Small-batch (latency) variant: groups of (query, deployment) pairs with
 // layer 2 split by columns over several blocks, plus quality blocks; scratch
 // pairC [Q][D], qualS [Q][M], h2 [Q D][H2], count [2 PAIRS_MAX_PAIRS] (query
@@ -154,7 +156,6 @@ cudaError_t launch_select_multi(const Model &m, const Queries &q, const float *C
                                 cudaStream_t s);
 int seq_chunk(const Model &m);
 size_t seq_table_floats(int D, int Qs);
-size_t route_simt_smem(const Model &m);
 size_t seq_table_smem(const Model &m);
 cudaError_t simt_prepare();   // one-time smem opt-in
 

@@ -27,6 +27,7 @@
 #include "hwr_internal.cuh"
 #include "select.cuh"
 #include "umma.cuh"
+#include "warp_tile.cuh"
 
 namespace hwr {
 
@@ -536,6 +537,415 @@ __global__ void __launch_bounds__(ROUTE_THREADS, CPT <= 4 ? 3 : 2) k_route_simt(
             q.util[qq] = ok ? best.U : __int_as_float(0x7fc00000);
         }
     }
+}
+
+// ---------------------------------------------------------------------------
+// K_route_rows: the fp32 kernel of large batches.  A block (one an SM) takes
+// an equal run of the batch's queries, in blocks of QBK (32, or 16 for more
+// than 32 deployments).  NW warps score their pairs in groups of RG rows with
+// the warp tile; NQ warps hold one query per lane and, a block of queries
+// ahead of the tile, run its quality chains, then wait for the block's costs
+// and decide.  The costs pass through a ring of NB blocks in shared memory
+// (mbarriers: done, a group's arrival; freed, the decision's), so the two
+// sides meet only when one is a whole ring ahead.
+// Bound: the FMA pipe; measured 42.5 TFLOP/s at 100,000 queries, D = 12,
+// H = 128 (53 % of 80.5; k_route_simt 31), where a k step's 64 packed FMAs
+// come with about 50 other instructions (the pairs of a W2 value with itself,
+// loads) and fill the issue slots.
+
+constexpr int QUAL_KC = 32;      // embedding elements per staged chunk
+constexpr int QUAL_MC = 16;      // model columns per staged chunk
+
+// Shape of the batch kernel by the width W of the layer-2 tile: rows per
+// group (lane tiles of 8 x 8, 8 x 4, 8 x 2 values), and 16 warps in all, so
+// that each thread can hold 128 registers.  Groups of 8 rows at W <= 128 read
+// more shared memory per FMA (1,048 against 969 us for 100,000 queries at
+// D = 12, H = 128), 16 at W = 256 need 16 x 8 lane tiles.
+template <int W>
+struct RouteShape {
+    static constexpr int RG = W == 256 ? 8 : 16;                 // rows per group
+    static constexpr int NQ = W <= 64 ? 4 : 2;                   // deciding warps
+    static constexpr int NW = 16 - NQ;                           // scoring warps
+    static constexpr int NB = NQ + 2;                            // query blocks in flight
+    static constexpr int NS = W <= 64 ? 8 : W == 128 ? 4 : 3;    // W2 stages at most
+    static constexpr int QST = 3;                                // embedding stages per deciding warp
+    static constexpr int THREADS = 32 * (NW + NQ);
+};
+
+constexpr size_t ROWS_SMEM = 227 * 1024;
+
+struct RowsLayout {
+    int qbk, cld, rowb, ns, nch;                     // query block, cost stride, embedding row bytes
+    size_t w2, bufs, ri, w1q, b2, w3, b3, cost, qst, qual, dms, bars, pre, total;   // bytes
+    bool pre_sm;                                     // the deployment prefixes in shared memory too
+    size_t qst_bytes;                                // one embedding stage
+};
+
+template <int W>
+__host__ __device__ inline RowsLayout rows_layout(int D, int M, int NH, int H1, int H2p, int es) {
+    using S = RouteShape<W>;
+    constexpr int RG = S::RG;
+    RowsLayout L;
+    L.qbk = D > 32 ? 16 : 32;
+    L.cld = D | 1;
+    L.rowb = QUAL_KC * es + 16;                      // an odd number of 16-byte units
+    L.nch = (H1 + TILE_KC - 1) / TILE_KC;
+    L.ns = L.nch < S::NS ? L.nch : S::NS;
+    L.qst_bytes = (size_t)L.qbk * L.rowb + (QUAL_KC + 1) * QUAL_MC * 4;
+    size_t o = 0;
+    auto take = [&o](size_t bytes) {
+        const size_t at = o;
+        o += (bytes + 15) & ~(size_t)15;
+        return at;
+    };
+    L.bufs = take((size_t)S::NW * Tile<W, RG>::BUF * 4);
+    L.ri = take((size_t)S::NW * RG * sizeof(RowInfo));
+    L.w1q = take(2 * (size_t)H1 * 4);
+    L.b2 = take(W * 4);
+    L.w3 = take((size_t)NH * H2p * 4);
+    L.b3 = take(16);
+    L.cost = take((size_t)S::NB * L.qbk * L.cld * 4);
+    L.qst = take((size_t)S::NQ * S::QST * L.qst_bytes);
+    L.qual = take((size_t)S::NQ * L.qbk * (M | 1) * 4);
+    L.dms = take((size_t)D * 4);
+    L.bars = take((S::NS + 2 * S::NB) * 8 + (S::NS + 2) * 4);
+    // W2 stages: as many as fit, all of it if possible (and slack: the widest
+    // lane reads past a row that ends before W)
+    const size_t stage = (size_t)TILE_KC * H2p * 4;
+    while (L.ns > 2 && o + L.ns * stage + W * 4 > ROWS_SMEM) --L.ns;
+    L.w2 = take(L.ns * stage + W * 4);
+    // the deployment prefixes where they fit: they are read once per row and
+    // 32 k (from global memory, a third of a group's time outside layer 2)
+    L.pre = o;
+    L.pre_sm = o + (size_t)D * H1 * 4 <= ROWS_SMEM;
+    if (L.pre_sm) take((size_t)D * H1 * 4);
+    L.total = o;
+    return L;
+}
+
+// One staged chunk of the quality chains of a query (row: its embedding,
+// mb: 4 NG of the staged model columns, rows of ms floats): KS elements'
+// operands at a time ahead of their FMAs.
+template <int NG>
+__device__ __forceinline__ void qual_chunk(const char *row, const float *mb, int ms, int kc, bool bf,
+                                           float (&acc)[QUAL_MC]) {
+    constexpr int KS = NG == 1 ? 8 : 4;
+#pragma unroll 1
+    for (int k = 0; k < kc; k += KS) {      // kc is a multiple of 8
+        float e[KS];
+        float4 b[KS][NG];
+        if (bf) {
+#pragma unroll
+            for (int i = 0; i < KS; i += 4) {
+                const uint2 t = *reinterpret_cast<const uint2 *>(row + 2 * (k + i));
+                e[i] = __uint_as_float(t.x << 16);
+                e[i + 1] = __uint_as_float(t.x & 0xffff0000u);
+                e[i + 2] = __uint_as_float(t.y << 16);
+                e[i + 3] = __uint_as_float(t.y & 0xffff0000u);
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < KS; i += 4) {
+                const float4 t = *reinterpret_cast<const float4 *>(row + 4 * (k + i));
+                e[i] = t.x;
+                e[i + 1] = t.y;
+                e[i + 2] = t.z;
+                e[i + 3] = t.w;
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < KS; ++i)
+#pragma unroll
+            for (int g = 0; g < NG; ++g)
+                b[i][g] = *reinterpret_cast<const float4 *>(mb + (k + i) * ms + 4 * g);
+#pragma unroll
+        for (int i = 0; i < KS; ++i)
+#pragma unroll
+            for (int g = 0; g < NG; ++g) {
+                acc[4 * g] = __fmaf_rn(e[i], b[i][g].x, acc[4 * g]);
+                acc[4 * g + 1] = __fmaf_rn(e[i], b[i][g].y, acc[4 * g + 1]);
+                acc[4 * g + 2] = __fmaf_rn(e[i], b[i][g].z, acc[4 * g + 2]);
+                acc[4 * g + 3] = __fmaf_rn(e[i], b[i][g].w, acc[4 * g + 3]);
+            }
+    }
+}
+
+template <int W>
+__global__ void __launch_bounds__(RouteShape<W>::THREADS, 1)
+k_route_rows(Model m, Queries q, int32_t *status) {
+    using S = RouteShape<W>;
+    constexpr int RG = S::RG, NW = S::NW, NQ = S::NQ, NB = S::NB, QST = S::QST;
+    extern __shared__ float4 sm4[];
+    char *sm = reinterpret_cast<char *>(sm4);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int D = m.D, M = m.M, F = m.F, H1 = m.H1, E = m.E;
+    const int es = q.emb_bf16 ? 2 : 4;
+    const RowsLayout L = rows_layout<W>(D, M, m.NH, H1, m.H2p, es);
+    const int QBK = L.qbk;
+    // this block's queries, their blocks, and the groups of a whole block
+    const int qa = (int)((long long)blockIdx.x * q.Q / gridDim.x);
+    const int qb = (int)((long long)(blockIdx.x + 1) * q.Q / gridDim.x);
+    const int nblk = (qb - qa + QBK - 1) / QBK;
+    const int G = (QBK * D + RG - 1) / RG;
+    const int last_groups = nblk ? ((qb - qa - (nblk - 1) * QBK) * D + RG - 1) / RG : 0;
+    const int ngroups = nblk ? (nblk - 1) * G + last_groups : 0;
+    const int passes = (ngroups + NW - 1) / NW;
+
+    uint64_t *full = reinterpret_cast<uint64_t *>(sm + L.bars), *done = full + S::NS,
+             *freed = done + NB;
+    uint32_t *used = reinterpret_cast<uint32_t *>(freed + NB);
+    volatile int *abort_f = reinterpret_cast<volatile int *>(used + S::NS);
+    W2Feed f;
+    f.w2t = m.W2T;
+    f.sm = reinterpret_cast<float *>(sm + L.w2);
+    f.full = full;
+    f.used = used;
+    f.issued = used + S::NS + 1;
+    f.abort_f = abort_f;
+    f.status = status;
+    f.H1 = H1;
+    f.ldw = m.H2p;
+    f.ns = L.ns;
+    f.nch = L.nch;
+    f.warps = NW;
+    f.total = (uint32_t)passes * L.nch;
+    if (tid == 0) {
+        for (int s = 0; s < S::NS; ++s) {
+            umma::mbar_init(&full[s], 1);
+            used[s] = 0;
+        }
+        for (int b = 0; b < NB; ++b) {
+            umma::mbar_init(&done[b], G);
+            umma::mbar_init(&freed[b], 1);
+        }
+        *abort_f = 0;
+        umma::fence_mbar_init();
+        w2_start(f);
+    }
+    TileWeights w;
+    uint32_t prefix_s = 0;
+    {
+        float *w1q = reinterpret_cast<float *>(sm + L.w1q), *b2 = reinterpret_cast<float *>(sm + L.b2);
+        float *w3 = reinterpret_cast<float *>(sm + L.w3), *b3 = reinterpret_cast<float *>(sm + L.b3);
+        int *dms = reinterpret_cast<int *>(sm + L.dms);
+        for (int k = tid; k < 2 * H1; k += S::THREADS) w1q[k] = m.W1T[(size_t)(F - 2) * H1 + k];
+        for (int n = tid; n < W; n += S::THREADS) b2[n] = n < m.H2 ? m.b2[n] : 0.f;
+        for (int i = tid; i < m.NH * m.H2; i += S::THREADS) {
+            const int o = i / m.H2;
+            w3[o * m.H2p + i - o * m.H2] = m.W3[i];
+        }
+        if (tid < m.NH) b3[tid] = m.b3[tid];
+        for (int d = tid; d < D; d += S::THREADS) dms[d] = m.dep_model[d];
+        if (L.pre_sm) {
+            float *pre = reinterpret_cast<float *>(sm + L.pre);
+            for (int i = tid; i < D * H1; i += S::THREADS) pre[i] = m.A[i];
+            prefix_s = umma::smem_u32(pre);
+        }
+        w.w1q = w1q;
+        w.b2 = b2;
+        w.w3 = w3;
+        w.b3 = b3;
+    }
+    __syncthreads();
+    float *costs = reinterpret_cast<float *>(sm + L.cost);
+
+    if (warp < NW) {
+        // ---- scoring warps --------------------------------------------------
+        float *buf = reinterpret_cast<float *>(sm + L.bufs) + (size_t)warp * Tile<W, RG>::BUF;
+        RowInfo *ri = reinterpret_cast<RowInfo *>(sm + L.ri) + RG * warp;
+        // lane l standardises slot l / RG (input, then output length) of row l % RG
+        const int r = lane % RG, slot_k = lane / RG == 1 ? F - 1 : F - 2;
+        const uint8_t xf = m.xform[slot_k];
+        const float mu = m.mu[slot_k], sd = m.sd[slot_k];
+        const float *lens = lane / RG == 1 ? q.out_len : q.in_len;
+        // row p of group g: its query and deployment (qq = -1 past the end)
+        auto row_of = [&](int g, int &qq, int &ql, int &d) {
+            const int blk = g / G, p = (g - blk * G) * RG + r;
+            ql = p / D;
+            d = p - ql * D;
+            qq = qa + blk * QBK + ql;
+            if (g >= ngroups || ql >= QBK || qq >= qb) qq = -1;
+        };
+        // the next group's lengths are loaded a group ahead
+        int qq, ql, d;
+        row_of(warp, qq, ql, d);
+        float len = qq < 0 ? 0.f : lens[qq];
+        for (int ps = 0, g = warp; ps < passes; ++ps, g += NW) {
+            const uint32_t n0 = (uint32_t)ps * (uint32_t)L.nch;
+            if (g >= ngroups) {
+                if (!w2_skip(f, n0)) break;
+                continue;
+            }
+            {
+                const float x = standardise(xf, len, mu, sd);
+                const float v = __shfl_down_sync(0xffffffffu, x, RG),
+                            ol = __shfl_down_sync(0xffffffffu, len, RG);
+                if (lane < RG) ri[lane] = RowInfo{x, v, qq < 0 ? 0 : d * H1, ol};
+            }
+            const int cq = qq, cql = ql, cd = d;
+            row_of(g + NW, qq, ql, d);
+            len = qq < 0 ? 0.f : lens[qq];
+            __syncwarp();
+            float C;
+            if (!warp_tile<W, RG>(m, f, w, n0, ri, m.A, prefix_s, buf, C)) break;
+            // the block's slot is free once the decisions NB blocks back are out
+            const int blk = g / G, slot = blk % NB;
+            if (blk >= NB) {
+                const bool ok = umma::mbar_wait(&freed[slot], ((blk / NB) & 1) ^ 1, abort_f, status);
+                if (!__all_sync(0xffffffffu, ok)) break;
+            }
+            if (lane < RG && cq >= 0) {
+                costs[(size_t)slot * QBK * L.cld + cql * L.cld + cd] = C;
+                if (q.pair_C) q.pair_C[(size_t)cq * D + cd] = C;
+            }
+            __syncwarp();
+            if (lane == 0) umma::mbar_arrive(&done[slot]);
+        }
+    } else {
+        // ---- deciding warps -------------------------------------------------
+        const int qw = warp - NW;
+        char *stages = sm + L.qst + (size_t)qw * QST * L.qst_bytes;
+        float *qs = reinterpret_cast<float *>(sm + L.qual) + (size_t)qw * QBK * (M | 1);
+        const int *dms = reinterpret_cast<const int *>(sm + L.dms);
+        const bool async = !q.inputs_host && ((uintptr_t)q.emb & 15) == 0;
+        const int ql = lane & (QBK - 1), nhalf = 32 / QBK, half = lane / QBK;
+        const int nck = (E + QUAL_KC - 1) / QUAL_KC, npass = (M + QUAL_MC - 1) / QUAL_MC;
+        const int myblk = nblk > qw ? (nblk - qw + NQ - 1) / NQ : 0;
+        const uint32_t stage_s = umma::smem_u32(stages);
+        // The next chunk (block nb, model pass np, k chunk nc, in order) into
+        // stage t % QST: the block's embedding rows and the pass's model columns;
+        // one cp.async group (empty past the last).  A lane copies granule ec of
+        // every er_step-th row.  Model columns: whole rows of M floats where M is
+        // at most 16 and a multiple of 4 (contiguous), else padded to 16.
+        const int gpr = QUAL_KC * es / 16, ec = lane & (gpr - 1), er0 = lane / gpr, er_step = 32 / gpr;
+        const bool mrow = M <= QUAL_MC && (M & 3) == 0;
+        const int ms = mrow ? M : QUAL_MC;
+        int nb = 0, np = 0, nc = 0;
+        auto issue = [&](int t) {
+            if (nb < myblk) {
+                const int k0 = nc * QUAL_KC, kc = min(QUAL_KC, E - k0), bq0 = qa + (qw + nb * NQ) * QBK;
+                const int nq = min(QBK, qb - bq0), m0 = np * QUAL_MC, mn = min(QUAL_MC, M - m0);
+                const size_t so = (size_t)(t % QST) * L.qst_bytes;
+                char *er = stages + so;
+                if (async) {
+                    if (ec * 16 < kc * es) {
+                        const char *src = (const char *)q.emb + ((size_t)(bq0 + er0) * E + k0) * es + 16 * ec;
+                        uint32_t dst = stage_s + (uint32_t)(so + (size_t)er0 * L.rowb + 16 * ec);
+                        for (int i = er0; i < nq; i += er_step) {
+                            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst),
+                                         "l"(__cvta_generic_to_global(src)) : "memory");
+                            src += (size_t)er_step * E * es;
+                            dst += (uint32_t)(er_step * L.rowb);
+                        }
+                    }
+                } else {
+                    for (int e = lane; e < nq * kc; e += 32) {
+                        const int i = e / kc, k = e - i * kc;
+                        const size_t src = (size_t)(bq0 + i) * E + k0 + k;
+                        if (es == 4) reinterpret_cast<float *>(er + (size_t)i * L.rowb)[k] = ((const float *)q.emb)[src];
+                        else reinterpret_cast<uint16_t *>(er + (size_t)i * L.rowb)[k] = ((const uint16_t *)q.emb)[src];
+                    }
+                }
+                const uint32_t mbs = stage_s + (uint32_t)(so + (size_t)QBK * L.rowb);
+                const float *mg = m.memb + (size_t)k0 * M + m0;
+                if (mrow) {
+                    for (int g = lane; g < kc * M / 4; g += 32)
+                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(mbs + 16u * g),
+                                     "l"(__cvta_generic_to_global(mg + 4 * g)) : "memory");
+                } else {
+                    for (int g = lane; g < kc * QUAL_MC; g += 32) {
+                        const int k = g / QUAL_MC, c = g % QUAL_MC;
+                        if (c < mn)
+                            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(mbs + 4u * g),
+                                         "l"(__cvta_generic_to_global(mg + (size_t)k * M + c)) : "memory");
+                    }
+                }
+                if (++nc == nck) {
+                    nc = 0;
+                    if (++np == npass) {
+                        np = 0;
+                        ++nb;
+                    }
+                }
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+        for (int t = 0; t < QST - 1; ++t) issue(t);
+        float acc[QUAL_MC];
+        int t = 0;
+        bool ok = true;
+        for (int bi = 0; ok && bi < myblk; ++bi) {
+            const int blk = qw + bi * NQ, slot = blk % NB, bq0 = qa + blk * QBK, nq = min(QBK, qb - bq0);
+            const int qq = bq0 + ql;
+            const bool valid = ql < nq;
+            for (int ps = 0; ps < npass; ++ps) {
+                const int m0 = ps * QUAL_MC, mn = min(QUAL_MC, M - m0);
+                const int ng = (mn + 4 * nhalf - 1) / (4 * nhalf);      // 4 model columns each
+                const int col = half * 4 * ng;
+#pragma unroll
+                for (int j = 0; j < QUAL_MC; ++j) acc[j] = 0.f;
+                for (int c = 0; c < nck; ++c, ++t) {
+                    asm volatile("cp.async.wait_group %0;" ::"n"(QST - 2) : "memory");
+                    __syncwarp();
+                    issue(t + QST - 1);
+                    const int kc = min(QUAL_KC, E - c * QUAL_KC);
+                    const char *er = stages + (size_t)(t % QST) * L.qst_bytes;
+                    const float *mb = reinterpret_cast<const float *>(er + (size_t)QBK * L.rowb) + col;
+                    const char *row = er + (size_t)ql * L.rowb;
+                    if (ng == 1) qual_chunk<1>(row, mb, ms, kc, es == 2, acc);
+                    else if (ng == 2) qual_chunk<2>(row, mb, ms, kc, es == 2, acc);
+                    else qual_chunk<4>(row, mb, ms, kc, es == 2, acc);
+                }
+#pragma unroll
+                for (int j = 0; j < QUAL_MC; ++j)
+                    if (j < 4 * ng && col + j < mn) {
+                        const float s = sigmoid_c(valid ? acc[j] : 0.f);
+                        qs[ql * (M | 1) + m0 + col + j] = s;
+                        if (q.qual_out && valid) q.qual_out[(size_t)qq * M + m0 + col + j] = s;
+                    }
+            }
+            __syncwarp();
+            // the groups that the last block does not have
+            if (blk == nblk - 1 && lane == 0)
+                for (int g = last_groups; g < G; ++g) umma::mbar_arrive(&done[slot]);
+            ok = umma::mbar_wait(&done[slot], (blk / NB) & 1, abort_f, status);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            // the decision: each lane its query's deployments in order (with 16
+            // queries: half of them), then the better half
+            const float slo = valid ? query_budget(q, qq) : 0.f;
+            const float *cr = costs + (size_t)slot * QBK * L.cld + ql * L.cld;
+            const float *qr = qs + ql * (M | 1);
+            Cand best = no_cand();
+            if (valid) {
+                const int d0 = half * D / nhalf, d1 = (half + 1) * D / nhalf;
+                for (int d = d0; d < d1; ++d) {
+                    const float C = cr[d], U = __fmaf_rn(-q.lam, C, __fmul_rn(q.wq, qr[dms[d]]));
+                    const Cand c = make_cand(C, U, d, slo);
+                    if (better(c, best)) best = c;
+                }
+            }
+            if (nhalf == 2) {
+                Cand o;
+                o.cls = __shfl_xor_sync(0xffffffffu, best.cls, 16);
+                o.d = __shfl_xor_sync(0xffffffffu, best.d, 16);
+                o.C = __shfl_xor_sync(0xffffffffu, best.C, 16);
+                o.U = __shfl_xor_sync(0xffffffffu, best.U, 16);
+                if (better(o, best)) best = o;
+            }
+            __syncwarp();
+            if (lane == 0) umma::mbar_arrive(&freed[slot]);
+            if (valid && half == 0) {
+                const bool sel = best.cls > 0;
+                q.chosen[qq] = sel ? best.d : -1;
+                q.lat[qq] = sel ? best.C : __int_as_float(0x7fc00000);
+                q.util[qq] = sel ? best.U : __int_as_float(0x7fc00000);
+            }
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+    }
+    __syncthreads();
+    if (tid == 0) w2_drain(f);
 }
 
 // ---------------------------------------------------------------------------
@@ -1587,10 +1997,6 @@ k_select_multi(Model m, Queries q, const float *C, const float *qual, int qstrid
 
 static int cpt_for(int H2) { return H2 <= 32 ? 1 : H2 <= 64 ? 2 : H2 <= 128 ? 4 : 8; }
 
-size_t route_simt_smem(const Model &m) {
-    return route_layout(m.D, m.M, m.H2).total * sizeof(float);
-}
-
 size_t seq_table_smem(const Model &m) {
     return seq_layout(m.H2).total * sizeof(float);
 }
@@ -1633,8 +2039,12 @@ static cudaError_t opt_in(K kernel, int bytes) {
 }
 
 cudaError_t simt_prepare() {
-    const int big = 200 * 1024;
+    const int big = 200 * 1024, most = 227 * 1024;
     cudaError_t e = cudaSuccess;
+    if (e == cudaSuccess) e = opt_in(k_route_rows<32>, most);
+    if (e == cudaSuccess) e = opt_in(k_route_rows<64>, most);
+    if (e == cudaSuccess) e = opt_in(k_route_rows<128>, most);
+    if (e == cudaSuccess) e = opt_in(k_route_rows<256>, most);
     if (e == cudaSuccess) e = opt_in(k_route_simt<1>, big);
     if (e == cudaSuccess) e = opt_in(k_route_simt<2>, big);
     if (e == cudaSuccess) e = opt_in(k_route_simt<4>, big);
@@ -1656,8 +2066,38 @@ cudaError_t launch_snapshot(const Model &m, const uint32_t *stage, cudaStream_t 
     return cudaGetLastError();
 }
 
-cudaError_t launch_route_simt(const Model &m, const Queries &q, cudaStream_t s) {
+template <int W>
+static cudaError_t launch_rows(const Model &m, const Queries &q, int nsm, int32_t *status,
+                               cudaStream_t s) {
+    const RowsLayout L = rows_layout<W>(m.D, m.M, m.NH, m.H1, m.H2p, q.emb_bf16 ? 2 : 4);
+    k_route_rows<W><<<q.Q < nsm ? q.Q : nsm, RouteShape<W>::THREADS, L.total, s>>>(m, q, status);
+    return cudaGetLastError();
+}
+
+// Which of the two batch kernels: k_route_rows once k_route_simt's blocks (64
+// rows; 3 an SM, 2 with more than 128 columns) would take more than one round.
+// Below that the fused blocks' short critical path wins, above it the tile
+// that keeps the FMA pipe busy.  Measured (us, simt / rows, E = 768 where not
+// said): H = 128, D = 12: 24,000 pairs 37.5 / 39.2, 36,000 49.5 / 49.5, 48,012
+// 68.0 / 55.4, 1.2 M 1,330 / 969; H = 128, D = 64: 32,000 62.7 / 53.6; H = 64:
+// 24,000 22.9 / 31.2, 48,000 39.4 / 36.9, 1.2 M 760 / 396; H = 32: 48,000
+// 31.4 / 33.1, 96,000 57.9 / 35.2, 1.2 M 610 / 236; H = 256: 18,000 71.2 /
+// 82.6, 30,000 134 / 103, 240,000 850 / 756.
+static bool rows_kernel(const Model &m, int Q, int nsm) {
+    return (long)Q * m.D > 64L * (m.H2 <= 128 ? 3 : 2) * nsm;
+}
+
+cudaError_t launch_route_simt(const Model &m, const Queries &q, int nsm, int32_t *status,
+                              cudaStream_t s) {
     if (q.Q <= 0) return cudaSuccess;
+    if (rows_kernel(m, q.Q, nsm)) {
+        switch (tile_width(m.H2)) {
+            case 32: return launch_rows<32>(m, q, nsm, status, s);
+            case 64: return launch_rows<64>(m, q, nsm, status, s);
+            case 128: return launch_rows<128>(m, q, nsm, status, s);
+            default: return launch_rows<256>(m, q, nsm, status, s);
+        }
+    }
     const RouteLayout L = route_layout(m.D, m.M, m.H2);
     const int blocks = (q.Q + L.QB - 1) / L.QB;
     const size_t smem = L.total * sizeof(float);

@@ -1,0 +1,111 @@
+"""The fp32 batch kernel of large batches (k_route_rows) against the oracle,
+bit for bit, at the sizes where it can go wrong: widths of the layer-2 tile
+and their remainders, K chunks resident and in the ring (H1 above four chunks
+at W = 128, three at W = 256), query blocks of 32 and 16 (D above 32) and
+their remainders, model columns staged as whole rows, padded, and in several
+passes, embedding tails, three heads, bf16 embeddings, unaligned device
+embeddings, and one query more or less than the batch size at which the
+kernel takes over."""
+import numpy as np
+import pytest
+
+import oracle as O
+import workload as W
+import paper_2608_14575_gb300 as H
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    H.build()
+
+
+def _problem(Q, M, G, H1, H2, E, dtype="f32", heads=2, seed=5):
+    return W.make_problem(Q=Q, M=M, G=G, F=M + G + 9 + seed % 4, H1=H1, H2=H2, E=E, dtype=dtype,
+                          lam=0.4, slo=3.0, seed=seed, bias_std=0.05, n_heads=heads)
+
+
+def _check(p, got, idx=None):
+    want = O.Problem(p).route(mode=O.F32, nthreads=16)
+    for g, w, t in zip(got, want, (np.int32, np.float32, np.float32)):
+        assert np.array_equal(np.asarray(g), np.asarray(w).astype(t), equal_nan=True)
+
+
+# (Q, M, G, H1, H2, E, dtype, heads): all above the take-over size
+CASES = [
+    (7500, 2, 2, 32, 32, 64, "f32", 2),
+    (5900, 5, 1, 17, 31, 40, "f32", 3),
+    (2433, 4, 3, 64, 33, 8, "f32", 2),
+    (4871, 3, 2, 50, 64, 96, "f32", 3),
+    (2440, 4, 3, 128, 128, 72, "f32", 2),
+    (1950, 5, 3, 129, 96, 104, "f32", 3),
+    (700, 9, 5, 160, 65, 64, "f32", 2),
+    (1470, 20, 1, 40, 128, 32, "f32", 2),
+    (900, 33, 1, 100, 70, 48, "f32", 3),
+    (1700, 4, 3, 200, 200, 64, "f32", 2),
+    (640, 8, 4, 256, 256, 64, "f32", 3),
+    (310, 16, 4, 96, 129, 136, "f32", 2),
+    (1000, 32, 1, 256, 64, 24, "f32", 2),
+    (480, 64, 1, 256, 100, 16, "f32", 3),
+    (1700, 4, 3, 200, 200, 64, "bf16", 2),
+    (650, 17, 2, 72, 136, 24, "bf16", 3),
+]
+
+
+@pytest.mark.parametrize("c", CASES, ids=lambda c: "-".join(map(str, c)))
+def test_large_batches_match_the_oracle(c):
+    p = _problem(*c)
+    r = H.Router(p)
+    _check(p, r.route(flags=H.HWR_PATH_SIMT))
+    r.close()
+
+
+@pytest.mark.parametrize("H2,per", [(128, 3), (160, 2)])
+def test_batches_around_the_take_over_size(H2, per):
+    import torch
+    nsm = torch.cuda.get_device_properties(0).multi_processor_count
+    D = 12
+    q0 = 64 * per * nsm // D
+    p = _problem(q0 + 2, 4, 3, 64, H2, 64)
+    r = H.Router(p)
+    for Q in (q0 - 1, q0, q0 + 1, q0 + 2):
+        s = W.query_slice(p, 0, Q)
+        _check(s, r.route(s["in_len"], s["out_len"], s["emb"]))
+    r.close()
+
+
+def test_budgets_scores_lambdas_and_unaligned_embeddings():
+    import torch
+    p = _problem(2500, 4, 3, 128, 128, 64)
+    st = torch.cuda.Stream()
+    r = H.Router(p, stream=st.cuda_stream)
+    orc = O.Problem(p)
+    Q, E = p["Q"], p["E"]
+    with torch.cuda.stream(st):
+        il, ol = (torch.from_numpy(p[k]).cuda() for k in ("in_len", "out_len"))
+        raw = torch.empty(Q * E + 1, device="cuda")
+        emb = raw[1:].view(Q, E)                       # 4-byte aligned only
+        emb.copy_(torch.from_numpy(p["emb"]))
+        out = [torch.empty(Q, dtype=t, device="cuda") for t in (torch.int32, torch.float32, torch.float32)]
+        cost, qual = torch.empty(Q, p["D"], device="cuda"), torch.empty(Q, p["M"], device="cuda")
+    st.synchronize()
+    r.route_device(il, ol, emb, *out, slo=p["slo"], lam=p["lam"])
+    _check(p, [o.cpu().numpy() for o in out])
+    r.score_device(il, ol, emb, cost, qual)
+    C, _ = orc.score_all(mode=O.F32, nthreads=16)
+    assert np.array_equal(cost.cpu().numpy(), C.astype(np.float32))
+    for i in range(0, Q, 97):
+        assert np.array_equal(qual[i].cpu().numpy(), orc.quality(p["emb"][i], mode=O.F32).astype(np.float32))
+    budgets = np.random.default_rng(3).lognormal(0.3, 0.8, Q).astype(np.float32)
+    budgets[::50] = np.nan
+    got = r.route_slo(budgets=budgets, lam=p["lam"])
+    want = orc.route_slo(budgets, p["in_len"], p["out_len"], p["emb"], mode=O.F32)
+    for g, w, t in zip(got, want, (np.int32, np.float32, np.float32)):
+        assert np.array_equal(g, np.asarray(w).astype(t), equal_nan=True)
+    lams = np.array([0.0, 0.2, 0.9], np.float32)
+    ch, lat, util = r.route_multi(lams)
+    for k, lam in enumerate(lams):
+        one = r.route(lam=float(lam))
+        assert all(np.array_equal(a[k], b) for a, b in zip((ch, lat, util), one))
+    r.close()
