@@ -1067,6 +1067,9 @@ static hwr_status route_impl(hwr_ctx *c, int32_t Q, const float *in_len, const f
     auto run_chunk = [&](Queries qc, int lo) -> hwr_status {
         const int n = qc.Q;
         const bool small = !tensor && (long)n * c->D <= c->pairs_max;
+        // the predictor kernel's own decisions are not wanted: the selection's
+        // replace them, or (scoring) there are none
+        if (tensor && (SC || SQ)) qc.no_select = 1;
         if (SC) qc.pair_C = SC + (size_t)lo * c->D;
         if (SQ) qc.qual_out = SQ + (size_t)lo * c->M;
         TRY(run_kernels(c, qc, flags, tensor));
@@ -1215,7 +1218,7 @@ extern "C" hwr_status hwr_route_batch_multi(hwr_ctx *c, int32_t Q, const float *
     if (!lambdas) return fail(c, HWR_ERR_INVALID_ARG, "lambdas is NULL");
     if (K < 1 || K > MAX_LAMBDAS)
         return fail(c, HWR_ERR_INVALID_ARG, "K=%d outside [1, %d]", K, MAX_LAMBDAS);
-    Lambdas L;
+    Lambdas L = {};
     L.K = K;
     for (int k = 0; k < K; ++k) {
         if (!isfinite(lambdas[k])) return fail(c, HWR_ERR_INVALID_ARG, "lambda %d not finite", k);

@@ -1942,53 +1942,135 @@ __global__ void __launch_bounds__(SIMT_THREADS) k_route_pairs(Model m, Queries q
 
 // ---------------------------------------------------------------------------
 // K_select_multi: the decision maker for several lambdas over stored scores.
-// One warp per query: lane l holds deployments l and l + 32 (D <= 64), loads
-// their costs and quality once, and for every lambda forms each candidate's
-// 40-bit key (the candidate order of the sequential chain, the same order as
-// make_cand / better) and takes the warp's largest with two 32-bit
-// reductions; lane k keeps lambda k's decision: 55 us for 8 lambdas over
-// 65,536 queries at D = 64 on GB300.  (A warp per (query, lambda), each with
-// its own warp reduction, took ~115 us; a thread per query with a running
-// best per lambda 99 us: too few warps, and divergent comparisons.)
+// SEL_LANES lanes per query: lane j scans every SEL_LANES-th group of four
+// deployments in order and keeps, for each of KT lambdas, the largest feasible
+// utility of a group and the group, and the smallest cost for the queries that
+// have no feasible deployment; the lanes' results are merged, and one lane per
+// lambda looks up the winner inside its group.  Bound: the ALU pipe (half the
+// FMA pipe's rate), so a (query, deployment, lambda) costs three FMA-pipe
+// instructions (an infeasible utility is pushed to -inf by an addition) and
+// one and a half ALU ones: 16 us for 8 lambdas over 65,536 queries
+// at D = 64 (a warp per query with two warp reductions per lambda took 53.5, a
+// compare and two selects per candidate 21).
+// Same order as make_cand / better: a feasible candidate is C <= SLO with a
+// defined utility; where a lambda has none, every defined cost is a candidate
+// of the other class, so the smallest cost serves all lambdas.
+constexpr int SEL_LANES = 4;
+
+template <int KT, bool VEC>
 __global__ void __launch_bounds__(SIMT_THREADS)
 k_select_multi(Model m, Queries q, const float *C, const float *qual, int qstride, Lambdas L,
                int ostride) {
-    const int qq = (blockIdx.x * SIMT_THREADS + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (qq >= q.Q) return;   // whole warps
-    const unsigned full = 0xffffffffu;
-    const float slo = query_budget(q, qq);
-    const int d0 = lane, d1 = lane + 32;
-    const bool h0 = d0 < m.D, h1 = d1 < m.D;
-    const float *cr = C + (size_t)qq * m.D, *qr = qual + (size_t)qq * qstride;
-    const float c0 = h0 ? cr[d0] : 0.f, c1 = h1 ? cr[d1] : 0.f;
-    const float g0 = h0 ? qr[m.dep_model[d0]] : 0.f, g1 = h1 ? qr[m.dep_model[d1]] : 0.f;
-    const float nan = __int_as_float(0x7fc00000);
-    int od = -1;
-    float oc = nan, ou = nan;
-    for (int k = 0; k < L.K; ++k) {
-        const float lam = L.lam[k], wq = L.wq[k];
-        const float u0 = __fmaf_rn(-lam, c0, __fmul_rn(wq, g0));
-        const float u1 = __fmaf_rn(-lam, c1, __fmul_rn(wq, g1));
-        const uint64_t k0 = h0 ? cand_key(c0, u0, d0, slo) : 0, k1 = h1 ? cand_key(c1, u1, d1, slo) : 0;
-        const uint64_t kl = k1 > k0 ? k1 : k0;
-        const uint32_t hi = __reduce_max_sync(full, (uint32_t)(kl >> 32));
-        const uint32_t lo = __reduce_max_sync(full, (uint32_t)(kl >> 32) == hi ? (uint32_t)kl : 0u);
-        const int wd = 63 - (int)(lo & 63u);
-        const bool ok = (hi >> 6) >= 2u;    // class feasible or infeasible, not NaN
-        // the winner's cost and utility, from the lane that holds it
-        const float wc = __shfl_sync(full, wd >= 32 ? c1 : c0, wd & 31);
-        const float wu = __shfl_sync(full, wd >= 32 ? u1 : u0, wd & 31);
-        if (lane == k) {
-            od = ok ? wd : -1;
-            oc = ok ? wc : nan;
-            ou = ok ? wu : nan;
+    __shared__ int dms[MAX_D + 4];
+    const int D = m.D;
+    for (int d = threadIdx.x; d < D; d += SIMT_THREADS) dms[d] = m.dep_model[d];
+    __syncthreads();
+    const int t = blockIdx.x * SIMT_THREADS + threadIdx.x, j = t % SEL_LANES;
+    const int qq = min(t / SEL_LANES, q.Q - 1);      // the last warp's spare lanes repeat the last query
+    const float slo = query_budget(q, qq), nan = __int_as_float(0x7fc00000);
+    const float inf = __int_as_float(0x7f800000);
+    const float *cr = C + (size_t)qq * D, *qr = qual + (size_t)qq * qstride;
+    float bu[KT], bc = nan;       // best utility per lambda, smallest cost
+    int bg[KT], bcd = -1;         // the group of bu (its first deployment), bc's deployment
+    bool any = false;             // a feasible cost
+#pragma unroll
+    for (int k = 0; k < KT; ++k) {
+        bu[k] = -inf;
+        bg[k] = 4 * j;
+    }
+    for (int d0 = 4 * j; d0 < D; d0 += 4 * SEL_LANES) {
+        float c[4], g[4], pen[4];
+        if constexpr (VEC) {
+            const float4 v = *reinterpret_cast<const float4 *>(cr + d0);
+            c[0] = v.x;
+            c[1] = v.y;
+            c[2] = v.z;
+            c[3] = v.w;
+        } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) c[i] = d0 + i < D ? cr[d0 + i] : nan;
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            g[i] = VEC || d0 + i < D ? qr[dms[d0 + i]] : 0.f;
+            pen[i] = c[i] <= slo ? 0.f : -inf;          // NaN costs too
+            any = any || c[i] <= slo;
+            // !(c >= bc): also when there is none yet; NaN costs never win
+            if (c[i] == c[i] && !(c[i] >= bc)) {
+                bc = c[i];
+                bcd = d0 + i;
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < KT; ++k) {
+            float u[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                u[i] = __fadd_rn(__fmaf_rn(-L.lam[k], c[i], __fmul_rn(L.wq[k], g[i])), pen[i]);
+            // (a NaN utility is no candidate, and fmaxf drops it)
+            const float best = fmaxf(fmaxf(u[0], u[1]), fmaxf(u[2], u[3]));
+            const bool win = best > bu[k];
+            bu[k] = win ? best : bu[k];
+            bg[k] = win ? d0 : bg[k];
         }
     }
-    if (lane < L.K) {
-        const size_t o = (size_t)lane * ostride + qq;
-        q.chosen[o] = od;
-        q.lat[o] = oc;
-        q.util[o] = ou;
+    const unsigned all = 0xffffffffu;
+#pragma unroll
+    for (int s = 1; s < SEL_LANES; s *= 2) {
+        const float oc = __shfl_xor_sync(all, bc, s);
+        const int ocd = __shfl_xor_sync(all, bcd, s);
+        if (ocd >= 0 && (bcd < 0 || oc < bc || (oc == bc && ocd < bcd))) {
+            bc = oc;
+            bcd = ocd;
+        }
+        any = __shfl_xor_sync(all, (int)any, s) || any;
+#pragma unroll
+        for (int k = 0; k < KT; ++k) {
+            const float ou = __shfl_xor_sync(all, bu[k], s);
+            const int og = __shfl_xor_sync(all, bg[k], s);
+            const bool win = ou > bu[k] || (ou == bu[k] && og < bg[k]);
+            bu[k] = win ? ou : bu[k];
+            bg[k] = win ? og : bg[k];
+        }
+    }
+    if (t / SEL_LANES >= q.Q) return;
+    // lane j finishes lambdas j, j + SEL_LANES, ...
+#pragma unroll
+    for (int k0 = 0; k0 < KT; k0 += SEL_LANES) {
+        float b = bu[k0];
+        int d0 = bg[k0];
+#pragma unroll
+        for (int i = 1; i < SEL_LANES; ++i) {
+            b = j == i ? bu[k0 + i] : b;
+            d0 = j == i ? bg[k0 + i] : d0;
+        }
+        const int k = k0 + j;
+        if (k >= L.K) continue;
+        const float lam = L.lam[k], wq = L.wq[k];
+        int bd = -1;
+        float cost = nan, u = nan;
+        if (any) {
+            // the first of the winning group's candidates with the best utility;
+            // a best of -inf may also be no group's: then all of them
+            const int d1 = b > -inf ? min(d0 + 4, D) : D;
+            for (int d = b > -inf ? d0 : 0; d < d1 && bd < 0; ++d) {
+                const float c = cr[d], v = __fmaf_rn(-lam, c, __fmul_rn(wq, qr[dms[d]]));
+                if (c <= slo && v == b) {
+                    bd = d;
+                    cost = c;
+                    u = v;
+                }
+            }
+        }
+        if (bd < 0 && bcd >= 0) {
+            bd = bcd;
+            cost = bc;
+            u = __fmaf_rn(-lam, bc, __fmul_rn(wq, qr[dms[bcd]]));
+        }
+        const size_t o = (size_t)k * ostride + qq;
+        q.chosen[o] = bd;
+        q.lat[o] = cost;
+        q.util[o] = u;
     }
 }
 
@@ -2151,9 +2233,19 @@ cudaError_t launch_select_multi(const Model &m, const Queries &q, const float *C
                                 const float *qual, int qstride, const Lambdas &L, int ostride,
                                 cudaStream_t s) {
     if (q.Q <= 0 || L.K <= 0 || L.K > MAX_LAMBDAS) return q.Q <= 0 || L.K <= 0 ? cudaSuccess : cudaErrorInvalidValue;
-    const long threads = (long)q.Q * 32;   // a warp per query
+    const long threads = (long)q.Q * SEL_LANES;
     const int blocks = (int)((threads + SIMT_THREADS - 1) / SIMT_THREADS);
-    k_select_multi<<<blocks, SIMT_THREADS, 0, s>>>(m, q, C, qual, qstride, L, ostride);
+    // rows of costs as 16-byte vectors where every row allows it
+    const bool vec = m.D % 4 == 0 && ((uintptr_t)C & 15) == 0;
+    const int kt = (L.K + 3) / 4;     // lambdas in fours (those past K are not written)
+#define HWR_SELECT(KT)                                                                              \
+    (vec ? k_select_multi<KT, true><<<blocks, SIMT_THREADS, 0, s>>>(m, q, C, qual, qstride, L, ostride) \
+         : k_select_multi<KT, false><<<blocks, SIMT_THREADS, 0, s>>>(m, q, C, qual, qstride, L, ostride))
+    if (kt == 1) HWR_SELECT(4);
+    else if (kt == 2) HWR_SELECT(8);
+    else if (kt == 3) HWR_SELECT(12);
+    else HWR_SELECT(16);
+#undef HWR_SELECT
     return cudaGetLastError();
 }
 
