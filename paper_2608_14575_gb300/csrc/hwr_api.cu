@@ -126,7 +126,7 @@ struct hwr_ctx {
     struct Range {
         const void *p = nullptr;
         size_t n = 0;
-    } prev_out[4];                   // chosen, latency, utility, per-pair costs
+    } prev_out[5];                   // chosen, latency, utility, per-pair costs, quality
     // a snapshot kernel may still read the staging: set at its launch, cleared
     // once the host has seen later work on the stream complete
     bool snap_busy = false;
@@ -824,22 +824,26 @@ static hwr_status run_kernels(hwr_ctx *c, const Queries &q, uint32_t flags, bool
         // and this call's inputs -- unless those inputs are outputs of the
         // previous tensor-core route, whose predictor may still be running.
         const size_t qb4 = (size_t)q.Q * 4;
-        bool early = true;
-        for (const auto &o : c->prev_out)
-            if (overlaps(q.in_len, qb4, o.p, o.n) || overlaps(q.out_len, qb4, o.p, o.n) ||
-                overlaps(q.emb, (size_t)q.Q * c->E * 2, o.p, o.n) ||
+        // (The quality kernel reads the embeddings at once: over earlier outputs
+        // it waits for the kernels before altogether.)
+        bool early = true, dependent = true;
+        for (const auto &o : c->prev_out) {
+            if (overlaps(q.emb, (size_t)q.Q * c->E * 2, o.p, o.n)) dependent = false;
+            if (!dependent || overlaps(q.in_len, qb4, o.p, o.n) || overlaps(q.out_len, qb4, o.p, o.n) ||
                 (q.slo_q && overlaps(q.slo_q, qb4, o.p, o.n)))
                 early = false;
+        }
         const int free_sms = tc_mlp_free_sms(q.Q, sp);
         LaunchScope a(c, HWR_K_QUAL_TC, prof);
-        CK(c, launch_qual_tc(t, q, qb, c->status_d, c->stream, true, early, free_sms, c->done_d,
-                             c->pred_ctas - c->pred_ctas_last),
+        CK(c, launch_qual_tc(t, q, qb, c->status_d, c->stream, dependent, early, free_sms, c->done_d,
+                             c->pred_ctas - c->pred_ctas_last, q.qual_out),
            "quality kernel");
         a.done();
         c->prev_out[0] = {q.chosen, qb4};
         c->prev_out[1] = {q.lat, qb4};
         c->prev_out[2] = {q.util, qb4};
         c->prev_out[3] = {q.pair_C, q.pair_C ? qb4 * c->D : 0};
+        c->prev_out[4] = {q.qual_out, q.qual_out ? qb4 * c->M : 0};
         LaunchScope b(c, HWR_K_MLP_TC, prof);
         int ctas = 0;
         CK(c, launch_mlp_tc(t, q, qb, sp, c->part, c->count, c->status_d, c->stream, c->done_d,
@@ -1056,9 +1060,11 @@ static hwr_status route_impl(hwr_ctx *c, int32_t Q, const float *in_len, const f
             SQ = so->quality;
         } else {
             TRY(grow(c, &c->mC, &c->mC_cap, (size_t)Q * c->D));
-            TRY(grow(c, &c->mQ, &c->mQ_cap, (size_t)Q * c->M));
             SC = c->mC;
-            SQ = c->mQ;
+            if (!(tensor && ml)) {
+                TRY(grow(c, &c->mQ, &c->mQ_cap, (size_t)Q * c->M));
+                SQ = c->mQ;
+            }
         }
     }
     const size_t rowC = (size_t)c->D * 4, rowQ = (size_t)c->M * 4;
@@ -1071,7 +1077,9 @@ static hwr_status route_impl(hwr_ctx *c, int32_t Q, const float *in_len, const f
         // replace them, or (scoring) there are none
         if (tensor && (SC || SQ)) qc.no_select = 1;
         if (SC) qc.pair_C = SC + (size_t)lo * c->D;
-        if (SQ) qc.qual_out = SQ + (size_t)lo * c->M;
+        // (the tensor path writes a scoring call's quality itself; a selection
+        // over several lambdas reads its scratch, rows of Mpad)
+        if (SQ && !(tensor && ml)) qc.qual_out = SQ + (size_t)lo * c->M;
         TRY(run_kernels(c, qc, flags, tensor));
         if (!SC && !SQ) return HWR_OK;
         // paths that keep their scores in their own scratch: copy them over
@@ -1081,19 +1089,9 @@ static hwr_status route_impl(hwr_ctx *c, int32_t Q, const float *in_len, const f
         if (small && SQ)
             CK(c, cudaMemcpyAsync(SQ + (size_t)lo * c->M, c->pairQ, n * rowQ,
                                   cudaMemcpyDeviceToDevice, c->stream), "copy quality");
-        // the selection over several lambdas reads the tensor path's quality
-        // buffer itself (rows of Mpad); only scoring copies it out
-        const float *selQ = SQ ? SQ + (size_t)lo * c->M : nullptr;
-        int qstride = c->M;
-        if (tensor && SQ && so)
-            CK(c, cudaMemcpy2DAsync(SQ + (size_t)lo * c->M, rowQ, c->qual_last, (size_t)c->Mpad * 4,
-                                    rowQ, n, cudaMemcpyDeviceToDevice, c->stream),
-               "copy quality");
-        if (tensor && SQ && !so) {
-            selQ = c->qual_last;
-            qstride = c->Mpad;
-        }
         if (!ml) return HWR_OK;
+        const float *selQ = tensor ? c->qual_last : SQ + (size_t)lo * c->M;
+        const int qstride = tensor ? c->Mpad : c->M;
         Queries qs = qc;
         qs.chosen = q.chosen + lo;
         qs.lat = q.lat + lo;
@@ -1338,6 +1336,7 @@ hwr_status hwr_internal_route_tensor_scratch(hwr_ctx *c, int32_t Q, const float 
     c->prev_out[1] = {pred_latency, qb4};
     c->prev_out[2] = {utility, qb4};
     c->prev_out[3] = {};
+    c->prev_out[4] = {};
     c->stats.kernel_launches++;
     c->stats.launches[HWR_K_MLP_TC]++;
     c->stats.queries_routed += Q;

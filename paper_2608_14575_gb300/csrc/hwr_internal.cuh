@@ -192,9 +192,12 @@ void tc_build_membimg(const uint16_t *memb_EM, int E, int M, int Mpad, int Epad,
 // after it leaves free (a small batch is spread over those alone).
 // done, done_target: the predictors' completion counter; before its first
 // store the grid waits for it to reach done_target (nullptr: no wait).
+// qual_out: the scores go to this [Q][M] array instead of `qual` (scoring calls,
+// whose predictor kernel reads no quality), once the kernel before has finished.
 cudaError_t launch_qual_tc(const TcModel &m, const Queries &q, float *qual,
                            int32_t *status, cudaStream_t s, bool dependent, bool early,
-                           int free_sms, const uint32_t *done, uint32_t done_target);
+                           int free_sms, const uint32_t *done, uint32_t done_target,
+                           float *qual_out = nullptr);
 // The first nwhole query tiles are processed whole; the deployments of each
 // remaining tile are split over nsplit units.  With nsplit > 1, `part`
 // (nsplit * Q records of 16 bytes) and `count` (Q int32, zero, self-resetting)

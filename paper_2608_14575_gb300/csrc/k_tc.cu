@@ -179,7 +179,7 @@ __device__ __forceinline__ float standardise_fast(uint8_t code, float v, float m
 
 __global__ void __launch_bounds__(QUAL_THREADS, 1)
 k_qual_tc(const __grid_constant__ CUtensorMap tmap, TcModel m, int Q, float *qual,
-          int32_t *status, int early, const uint32_t *done, uint32_t done_target) {
+          int32_t *status, int early, const uint32_t *done, uint32_t done_target, float *qual_out) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *sm = align1024(smem_raw);
     const QualLayout L = qual_layout(m.Mpad, m.Epad);
@@ -303,7 +303,13 @@ k_qual_tc(const __grid_constant__ CUtensorMap tmap, TcModel m, int Q, float *qua
             }
             tc_fence_before();
             mbar_arrive(&acce[b]);
-            if (!may_store) {
+            if (qual_out) {
+                // The caller's array: the kernel before may still write it (the
+                // quality kernel of a call before, which that predictor waits
+                // for), so nothing is stored before it has finished.  Two tiles
+                // a block are computed by then.
+                if (lt == 0) grid_dependency_wait();
+            } else if (!may_store) {
                 // This buffer was last read by the predictor two routes back
                 // (the buffers alternate), which may still run when this grid
                 // starts: before the first store, every predictor CTA launched
@@ -316,14 +322,25 @@ k_qual_tc(const __grid_constant__ CUtensorMap tmap, TcModel m, int Q, float *qua
             }
             const int row = t * BM + r;
             if (row < Q) {
-                float4 *dst = (float4 *)(qual + (size_t)row * Mpad);
-                for (int i = 0; i < Mpad; i += 4) {
+                // rows of Mpad in the scratch, or of M in the caller's array
+                // (vectors where its rows allow them)
+                const int ld = qual_out ? m.M : Mpad;
+                float *dst = (qual_out ? qual_out : qual) + (size_t)row * ld;
+                const bool vec = (ld & 3) == 0 && ((uintptr_t)dst & 15) == 0;
+                for (int i = 0; i < ld; i += 4) {
                     float4 o;
                     o.x = i + 0 < m.M ? 1.f / (1.f + expf(-__uint_as_float(v[i + 0]))) : 0.f;
                     o.y = i + 1 < m.M ? 1.f / (1.f + expf(-__uint_as_float(v[i + 1]))) : 0.f;
                     o.z = i + 2 < m.M ? 1.f / (1.f + expf(-__uint_as_float(v[i + 2]))) : 0.f;
                     o.w = i + 3 < m.M ? 1.f / (1.f + expf(-__uint_as_float(v[i + 3]))) : 0.f;
-                    dst[i >> 2] = o;
+                    if (vec) {
+                        *(float4 *)(dst + i) = o;
+                    } else {
+                        dst[i] = o.x;
+                        if (i + 1 < ld) dst[i + 1] = o.y;
+                        if (i + 2 < ld) dst[i + 2] = o.z;
+                        if (i + 3 < ld) dst[i + 3] = o.w;
+                    }
                 }
             }
         }
@@ -586,7 +603,7 @@ k_mlp_tc(TcModel m, Queries q, const __grid_constant__ HeadConsts hc,
             const float ol = valid ? q.out_len[row] : 0.f;
             const float slo_r = valid ? query_budget(q, row) : slo;
             for (int i = 0; i < m.M; ++i)
-                qs[r * QS + i] = valid ? qual[(size_t)row * Mpad + i] : 0.f;
+                qs[r * QS + i] = valid && !q.no_select ? qual[(size_t)row * Mpad + i] : 0.f;
             Cand best = no_cand();
             for (int d = un.d0; d < un.d1; ++d, ++g) {
                 const int b = g & 1;
@@ -896,7 +913,7 @@ cudaError_t tc_prepare() {
 
 cudaError_t launch_qual_tc(const TcModel &m, const Queries &q, float *qual, int32_t *status,
                            cudaStream_t s, bool dependent, bool early, int free_sms,
-                           const uint32_t *done, uint32_t done_target) {
+                           const uint32_t *done, uint32_t done_target, float *qual_out) {
     if (q.Q <= 0) return cudaSuccess;
     CUtensorMap map;
     const cuuint64_t dims[2] = {(cuuint64_t)m.E, (cuuint64_t)q.Q};
@@ -935,7 +952,7 @@ cudaError_t launch_qual_tc(const TcModel &m, const Queries &q, float *qual, int3
     cfg.attrs = at;
     cfg.numAttrs = dependent ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, k_qual_tc, map, m, q.Q, qual, status, early ? 1 : 0, done,
-                              done_target);
+                              done_target, qual_out);
 }
 
 cudaError_t launch_mlp_tc_scores(const TcModel &m, const Queries &q, const float *qual,
