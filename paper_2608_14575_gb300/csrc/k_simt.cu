@@ -1165,32 +1165,20 @@ k_seq_table(Model m, Queries q, int Qs, int nb_qual, int rows_per_block, float *
     }
 }
 
-// Chain shared memory (4-byte words): dep_model and picks [MAX_D] ints each,
-// the table [T rounded up to 4] (16-byte aligned), the chunk's quality
-// [Qs][M], budgets [Qs] and the walk's outputs (chosen, latency, utility)
-// [3][Qs].
+// Chain shared memory (4-byte words): dep_model and picks per deployment
+// [MAX_D] ints each, the walk's picks [SEQ_MAX_CHUNK], the table [T rounded up
+// to 4] (16-byte aligned), the chunk's quality [Qs][M] and budgets [Qs].
 constexpr int CHAIN_THREADS = 1024;
 
 __host__ __device__ inline size_t chain_tab_floats(int D, int Qs) {
     return (tri_off(D, Qs, Qs) + 3) & ~(size_t)3;
 }
 
-// The decision maker's candidate order as one 40-bit integer: class + 1
-// (bits 38-39), the key within the class (bits 6-37: larger U for a
-// feasible candidate, smaller C for an infeasible one, as order-preserving
-// integers) and 63 - d (bits 0-5), so that the largest value is the best
-// candidate and ties go to the lowest deployment.  Same classes as make_cand.
-// Written with selects only: the walk is one warp's dependent chain, and a
-// divergent branch there costs more than the few extra instructions.
-__device__ __forceinline__ uint64_t cand_key(float C, float U, int d, float slo) {
-    const bool nan = C != C;
-    const bool feas = C <= slo && U == U;       // false for a NaN cost
-    const uint32_t kU = order_key(U), kC = ~order_key(C);
-    uint32_t key = feas ? kU : kC, cls = feas ? 3u : 2u;
-    key = nan ? 1u : key;
-    cls = nan ? 1u : cls;
-    const uint32_t hi = (cls << 6) | (key >> 26), lo = (key << 6) | (uint32_t)(63 - d);
-    return ((uint64_t)hi << 32) | lo;
+// Largest value over a full warp (NaN lanes do not count).
+__device__ __forceinline__ float warp_max(float x) {
+    float r;
+    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
+    return r;
 }
 
 // HI: deployments 32 .. 63 exist (D > 32); without them every lane of the
@@ -1207,20 +1195,18 @@ k_seq_chain(Model m, Queries q, int Qs, const float *ctab, float *aux, const flo
     const int D = m.D, M = m.M, F = m.F, H1 = m.H1, P = m.P;
     const SeqAux A = seq_aux(aux, D, M, Qs);
     const size_t T = tri_off(D, Qs, Qs);
-    int *dm = reinterpret_cast<int *>(sm), *cnt = dm + MAX_D;
-    float *tab = sm + 2 * MAX_D;
+    int *dm = reinterpret_cast<int *>(sm), *cnt = dm + MAX_D, *o_ch = cnt + MAX_D;
+    float *tab = sm + 2 * MAX_D + SEQ_MAX_CHUNK;
     float *qs = tab + (BIG ? (size_t)tsm : chain_tab_floats(D, Qs)), *slo = qs + (size_t)Qs * M;
     const size_t Ts = BIG ? (size_t)tsm : T;    // entries staged in shared memory
     // entry e of the table: shared memory, or (BIG, e >= tsm) global memory
     auto at = [&](int e) -> float {
         if constexpr (BIG) {
-            return e < tsm ? tab[e] : __ldcg(ctab + e);
+            return e < tsm ? tab[e] : __ldcg(ctab + (e < (int)T ? e : (int)T - 1));
         } else {
             return tab[e];
         }
     };
-    float *o_lat = slo + Qs, *o_util = o_lat + Qs;
-    int *o_ch = reinterpret_cast<int *>(o_util + Qs);
 
     // launched as a programmatic dependent of the table kernel: budgets and
     // the model map first, then wait for the table (and, through it, for the
@@ -1245,116 +1231,185 @@ k_seq_chain(Model m, Queries q, int Qs, const float *ctab, float *aux, const flo
     __syncthreads();
 
     if (tid < 32) {
-        // The walk.  Lane l holds deployments d0 = l and d1 = l + 32 with their
-        // picks so far (c0, c1); entry (c, d, i) is tab[tab_row(c, d) + i].
+        // The walk.  Lane l holds deployments d0 = l and d1 = l + 32; entry
+        // (c, d, i) is tab[tab_row(c, d) + i], c the deployment's picks so far.
         // While step i is decided, step i + 1's entries at the current count
-        // and at one more pick are loaded and turned into candidate keys, so a
-        // step is a choice between two ready keys, a 64-bit max over the warp
-        // (two reductions) and the winner's index from the low bits.  Lanes
-        // without a deployment shadow deployment D - 1 (valid addresses) and
-        // keep key 0, below every candidate; the row of one more pick advances
-        // by D (Qs - c) - d - 1 after a pick.  The step has no branch: the last
-        // step loads its own column again (valid entries, unused), and a pick
-        // moves the rows by selects.
-        const unsigned full = 0xffffffffu;
+        // and at one more pick are loaded and made candidates, so a step is two
+        // float maxima over the warp (the feasible utilities; the costs, for a
+        // step without a feasible deployment), one vote, the lowest lane that
+        // holds the maximum, and a choice between two ready candidates.  It is
+        // one chain of dependent instructions, and each one on it counts: no
+        // find-first-set (a lane asks its lane mask), no store, no branch; only
+        // the picks are kept (lane i % 32 keeps step i's), the outputs follow
+        // from them below.  A step takes ~145 cycles at D = 12 and ~255 at
+        // D = 32 with part of the table in L2; with 40-bit integer keys, stores
+        // and branches 260 and 411, the walk of a 64-request chunk 8.0 -> 4.5 us.
+        // Exact while the costs met and the weights are ordinary numbers: then a
+        // utility is finite, and the maximum is -inf only if nothing is
+        // feasible.  Otherwise the walk runs again the long way.
+        // Lanes without a deployment shadow deployment D - 1 (valid addresses)
+        // and are no candidates.  The last step loads a column past the end: the
+        // row after, or the value behind the table (both unused).
+        const unsigned full = 0xffffffffu, below = (1u << lane) - 1u;
+        const float ninf = __int_as_float(0xff800000), pinf = __int_as_float(0x7f800000);
         const int d0 = lane, d1 = lane + 32;
         const bool h0 = d0 < D, h1 = HI && d1 < D;
         const int e0 = h0 ? d0 : D - 1, e1 = h1 ? d1 : D - 1;
         const int m0 = dm[e0], m1 = HI ? dm[e1] : 0;
         const float lam = q.lam, wq = q.wq;
-        int c0 = 0, c1 = 0;
-        int r0 = tab_row(D, Qs, 0, e0), r1 = HI ? tab_row(D, Qs, 0, e1) : 0;
-        int r0p = r0 + D * Qs - e0 - 1, r1p = HI ? r1 + D * Qs - e1 - 1 : 0;
-        // this step's candidate of each deployment: cost, utility, key
-        float C0, U0, C1 = 0.f, U1 = 0.f;
-        uint64_t K0, K1 = 0;
-        {
-            const float b = slo[0];
-            C0 = at(r0);
-            U0 = __fmaf_rn(-lam, C0, __fmul_rn(wq, qs[m0]));
-            K0 = cand_key(C0, U0, d0, b);
-            K0 = h0 ? K0 : 0;
-            if (HI) {
-                C1 = at(r1);
-                U1 = __fmaf_rn(-lam, C1, __fmul_rn(wq, qs[m1]));
-                K1 = cand_key(C1, U1, d1, b);
-                K1 = h1 ? K1 : 0;
+        // a candidate: minus its cost, and its utility if feasible (a NaN there
+        // is never the maximum)
+        struct Entry {
+            float n, v;
+        };
+        auto entry = [&](float C, float wQ, float b, bool h) -> Entry {
+            return Entry{h ? -C : ninf, h && C <= b ? __fmaf_rn(-lam, C, wQ) : ninf};
+        };
+        // next column's entry at this count and at one more; the latter's row
+        // moves on by s = D (Qs - c) - d - 1 with each pick
+        int a0, a1, s0, s1, a0p, a1p;
+        const float *qn0, *qn1;
+        Entry E0, E1;
+        auto start = [&]() {
+            a0 = tab_row(D, Qs, 0, e0);
+            a1 = HI ? tab_row(D, Qs, 0, e1) : 0;
+            s0 = D * Qs - e0 - 1;
+            s1 = D * Qs - e1 - 1;
+            E0 = entry(at(a0), __fmul_rn(wq, qs[m0]), slo[0], h0);
+            E1 = E0;
+            if (HI) E1 = entry(at(a1), __fmul_rn(wq, qs[m1]), slo[0], h1);
+            ++a0;
+            ++a1;
+            a0p = a0 + s0;
+            a1p = a1 + s1;
+            qn0 = qs + m0;
+            qn1 = qs + m1;
+        };
+        // one step's state from its decision
+        auto advance = [&](bool p, const Entry &es, const Entry &ep, Entry &e, int &ac, int &ap, int &st) {
+            e.n = p ? ep.n : es.n;
+            e.v = p ? ep.v : es.v;
+            st -= p ? D : 0;
+            ac = (p ? ap : ac) + 1;
+            ap += (p ? st : 0) + 1;
+        };
+        bool odd = !(fabsf(lam) <= 1e6f && fabsf(wq) <= 1e6f);
+        // steps lo .. hi - 1 (at most 32); lane i % 32 keeps step i's votes
+        auto steps = [&](int lo, int hi, uint32_t &rec0, uint32_t &rec1) {
+#pragma unroll 2
+            for (int i = lo; i < hi; ++i) {
+                const bool more = i + 1 < Qs;
+                const float b = slo[more ? i + 1 : i];
+                qn0 += more ? M : 0;
+                const float q0 = *qn0, x0s = at(a0), x0p = at(a0p);
+                float q1 = 0.f, x1s = 0.f, x1p = 0.f;
+                if (HI) {
+                    qn1 += more ? M : 0;
+                    q1 = *qn1;
+                    x1s = at(a1);
+                    x1p = at(a1p);
+                }
+                const float mx = warp_max(HI ? fmaxf(E0.v, E1.v) : E0.v);
+                const float mn = warp_max(HI ? fmaxf(E0.n, E1.n) : E0.n);
+                const bool feas = mx > ninf;
+                const bool k0 = feas ? E0.v == mx : E0.n == mn;
+                const bool k1 = HI && (feas ? E1.v == mx : E1.n == mn);
+                const unsigned w0 = __ballot_sync(full, k0), w1 = HI ? __ballot_sync(full, k1) : 0u;
+                const bool p0 = k0 && (w0 & below) == 0u, p1 = HI && k1 && (w0 | (w1 & below)) == 0u;
+                odd = odd || (h0 && !(fabsf(E0.n) <= 1e30f)) || (h1 && !(fabsf(E1.n) <= 1e30f));
+                rec0 = lane == (i & 31) ? w0 : rec0;
+                if (HI) rec1 = lane == (i & 31) ? w1 : rec1;
+                const float wQ0 = __fmul_rn(wq, q0);
+                advance(p0, entry(x0s, wQ0, b, h0), entry(x0p, wQ0, b, h0), E0, a0, a0p, s0);
+                if (HI) {
+                    const float wQ1 = __fmul_rn(wq, q1);
+                    advance(p1, entry(x1s, wQ1, b, h1), entry(x1p, wQ1, b, h1), E1, a1, a1p, s1);
+                }
+            }
+        };
+        start();
+        uint32_t ra0 = 0u, ra1 = 0u, rb0 = 0u, rb1 = 0u;
+        steps(0, min(Qs, 32), ra0, ra1);
+        steps(32, Qs, rb0, rb1);
+        if (lane < Qs) o_ch[lane] = ra0 ? __ffs(ra0) - 1 : 31 + __ffs(ra1);
+        if (lane + 32 < Qs) o_ch[lane + 32] = rb0 ? __ffs(rb0) - 1 : 31 + __ffs(rb1);
+        if (__any_sync(full, odd)) {
+            __syncwarp();
+            start();
+#pragma unroll 1
+            for (int i = 0; i < Qs; ++i) {
+                const bool more = i + 1 < Qs;
+                const float b = slo[more ? i + 1 : i], bi = slo[i];
+                qn0 += more ? M : 0;
+                qn1 += HI && more ? M : 0;
+                const float x0s = at(a0), x0p = at(a0p), x1s = HI ? at(a1) : 0.f, x1p = HI ? at(a1p) : 0.f;
+                // the classes in turn: feasible with a defined utility (-inf among
+                // them), any defined cost, none
+                const float C0 = -E0.n, C1 = -E1.n;
+                const bool f0 = h0 && C0 <= bi && E0.v == E0.v, f1 = h1 && C1 <= bi && E1.v == E1.v;
+                const float mx = warp_max(HI ? fmaxf(f0 ? E0.v : ninf, f1 ? E1.v : ninf) : f0 ? E0.v : ninf);
+                bool k0 = f0 && E0.v == mx, k1 = f1 && E1.v == mx;
+                unsigned w0 = __ballot_sync(full, k0), w1 = __ballot_sync(full, k1);
+                if ((w0 | w1) == 0u) {
+                    const bool n0 = h0 && C0 == C0, n1 = h1 && C1 == C1;
+                    const float mn = warp_max(fmaxf(n0 ? E0.n : ninf, n1 ? E1.n : ninf));
+                    k0 = n0 && E0.n == mn;
+                    k1 = n1 && E1.n == mn;
+                    w0 = __ballot_sync(full, k0);
+                    w1 = __ballot_sync(full, k1);
+                }
+                if (lane == 0) o_ch[i] = w0 ? __ffs(w0) - 1 : w1 ? 31 + __ffs(w1) : -1;
+                const bool p0 = k0 && (w0 & below) == 0u, p1 = k1 && (w0 | (w1 & below)) == 0u;
+                const float wQ0 = __fmul_rn(wq, *qn0);
+                advance(p0, entry(x0s, wQ0, b, h0), entry(x0p, wQ0, b, h0), E0, a0, a0p, s0);
+                if (HI) {
+                    const float wQ1 = __fmul_rn(wq, *qn1);
+                    advance(p1, entry(x1s, wQ1, b, h1), entry(x1p, wQ1, b, h1), E1, a1, a1p, s1);
+                }
             }
         }
-        for (int i = 0; i < Qs; ++i) {
-            // step j = i + 1's candidates: s = same count, p = after one more
-            // pick (at the last step, j = i: this step's entries again)
-            const bool more = i + 1 < Qs;
-            const int j = more ? i + 1 : i;
-            const float b = slo[j];
-            const float wQ0 = __fmul_rn(wq, qs[j * M + m0]);
-            const float C0s = at(r0 + j), C0p = at((more ? r0p : r0) + j);
-            const float U0s = __fmaf_rn(-lam, C0s, wQ0), U0p = __fmaf_rn(-lam, C0p, wQ0);
-            uint64_t K0s = cand_key(C0s, U0s, d0, b), K0p = cand_key(C0p, U0p, d0, b);
-            K0s = h0 ? K0s : 0;
-            K0p = h0 ? K0p : 0;
-            float C1s = 0.f, U1s = 0.f, C1p = 0.f, U1p = 0.f;
-            uint64_t K1s = 0, K1p = 0;
-            if (HI) {
-                const float wQ1 = __fmul_rn(wq, qs[j * M + m1]);
-                C1s = at(r1 + j);
-                C1p = at((more ? r1p : r1) + j);
-                U1s = __fmaf_rn(-lam, C1s, wQ1);
-                U1p = __fmaf_rn(-lam, C1p, wQ1);
-                K1s = cand_key(C1s, U1s, d1, b);
-                K1p = cand_key(C1p, U1p, d1, b);
-                K1s = h1 ? K1s : 0;
-                K1p = h1 ? K1p : 0;
-            }
-            // step i: the warp's largest key
-            const uint64_t kl = HI && K1 > K0 ? K1 : K0;
-            const uint32_t hi = __reduce_max_sync(full, (uint32_t)(kl >> 32));
-            const uint32_t lo =
-                __reduce_max_sync(full, (uint32_t)(kl >> 32) == hi ? (uint32_t)kl : 0u);
-            const int wd = 63 - (int)(lo & 63u);
-            const bool ok = (hi >> 6) >= 2u;    // class feasible or infeasible, not NaN
-            const bool p0 = ok && wd == d0, p1 = HI && ok && wd == d1;
-            if (lane == 0) o_ch[i] = ok ? wd : -1;
-            if (p0 || p1) {
-                o_lat[i] = p0 ? C0 : C1;
-                o_util[i] = p0 ? U0 : U1;
-            }
-            if (!ok && lane == 0) {
-                o_lat[i] = __int_as_float(0x7fc00000);
-                o_util[i] = __int_as_float(0x7fc00000);
-            }
-            c0 += p0 ? 1 : 0;
-            const int n0 = r0p + D * (Qs - c0) - e0 - 1;
-            r0 = p0 ? r0p : r0;
-            r0p = p0 ? n0 : r0p;
-            C0 = p0 ? C0p : C0s;
-            U0 = p0 ? U0p : U0s;
-            K0 = p0 ? K0p : K0s;
-            if (HI) {
-                c1 += p1 ? 1 : 0;
-                const int n1 = r1p + D * (Qs - c1) - e1 - 1;
-                r1 = p1 ? r1p : r1;
-                r1p = p1 ? n1 : r1p;
-                C1 = p1 ? C1p : C1s;
-                U1 = p1 ? U1p : U1s;
-                K1 = p1 ? K1p : K1s;
-            }
-        }
-        if (h0) cnt[d0] = c0;
-        if (h1) cnt[d1] = c1;
     }
     __syncthreads();
-    for (int i = tid; i < Qs; i += CHAIN_THREADS) {
-        q.lat[i] = o_lat[i];
-        q.util[i] = o_util[i];
-        if (q.inputs_host) {
-            // outputs in host memory: the host may poll chosen with acquire
-            // loads, so it is stored last, with release semantics at system
-            // scope
-            asm volatile("st.release.sys.global.b32 [%0], %1;" ::"l"(q.chosen + i), "r"(o_ch[i])
-                         : "memory");
-        } else {
-            q.chosen[i] = o_ch[i];
+    // The outputs of step i: its pick's count is the number of earlier steps
+    // that picked the same deployment.  Sixteen threads a step (and as many a
+    // deployment, for its picks in all) look at four picks each.
+    static_assert(CHAIN_THREADS == 16 * SEQ_MAX_CHUNK && MAX_D == SEQ_MAX_CHUNK, "sixteen threads a step");
+    {
+        const int i = tid / 16, j0 = 4 * (tid % 16);
+        const int4 v = *reinterpret_cast<const int4 *>(o_ch + j0);   // (past the picks: never counted)
+        const int pick[4] = {v.x, v.y, v.z, v.w};
+        const int d = i < Qs ? o_ch[i] : -1;
+        int c = 0, all = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            c += pick[k] == d && j0 + k < i ? 1 : 0;
+            all += pick[k] == i && j0 + k < Qs ? 1 : 0;      // this group's deployment is i too
+        }
+#pragma unroll
+        for (int s = 8; s; s >>= 1) {
+            c += __shfl_xor_sync(0xffffffffu, c, s);
+            all += __shfl_xor_sync(0xffffffffu, all, s);
+        }
+        if (tid % 16 == 0) {
+            cnt[i] = all;
+            if (i < Qs) {
+                float C = __int_as_float(0x7fc00000), U = C;
+                if (d >= 0) {
+                    C = at(tab_row(D, Qs, c, d) + i);
+                    U = __fmaf_rn(-q.lam, C, __fmul_rn(q.wq, qs[i * M + dm[d]]));
+                }
+                q.lat[i] = C;
+                q.util[i] = U;
+                if (q.inputs_host) {
+                    // outputs in host memory: the host may poll chosen with
+                    // acquire loads, so it is stored last, with release
+                    // semantics at system scope
+                    asm volatile("st.release.sys.global.b32 [%0], %1;" ::"l"(q.chosen + i), "r"(d)
+                                 : "memory");
+                } else {
+                    q.chosen[i] = d;
+                }
+            }
         }
     }
     __syncthreads();
@@ -2084,7 +2139,7 @@ size_t seq_table_smem(const Model &m) {
 }
 
 static size_t chain_smem(int D, int M, int Qs) {
-    return (2 * MAX_D + chain_tab_floats(D, Qs) + (size_t)Qs * M + 4 * (size_t)Qs) * sizeof(float);
+    return (2 * MAX_D + SEQ_MAX_CHUNK + chain_tab_floats(D, Qs) + (size_t)Qs * M + (size_t)Qs) * sizeof(float);
 }
 
 
