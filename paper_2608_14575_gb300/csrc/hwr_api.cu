@@ -785,7 +785,7 @@ static hwr_status run_kernels(hwr_ctx *c, const Queries &q, uint32_t flags, bool
                 c->pred_ctas += (uint32_t)ctas;
                 c->pred_ctas_last = (uint32_t)ctas;
                 a.done();
-                CK(c, launch_seq_chain_tc(m, k, n, c->ctab, c->qseq, qb, c->Mpad, c->stream),
+                CK(c, launch_seq_chain_tc(m, k, n, c->ctab, c->qseq, qb, c->Mpad, lo + Qs < q.Q, c->stream),
                    "sequential chain");
                 // preparation, quality and chain beside the scope's table kernel
                 c->stats.kernel_launches += 3;
@@ -796,7 +796,8 @@ static hwr_status run_kernels(hwr_ctx *c, const Queries &q, uint32_t flags, bool
             CK(c, launch_seq_table(m, k, n, c->seq_slots, c->ctab, c->qseq, c->stream),
                "sequential table");
             a.done();
-            CK(c, launch_seq_chain(m, k, n, c->ctab, c->qseq, c->stream), "sequential chain");
+            CK(c, launch_seq_chain(m, k, n, c->ctab, c->qseq, lo + Qs < q.Q, c->stream),
+               "sequential chain");
             // the preparation kernel (inside launch_seq_table) and the chain
             c->stats.kernel_launches += 2;
             c->stats.launches[HWR_K_SEQ_TABLE] += 2;

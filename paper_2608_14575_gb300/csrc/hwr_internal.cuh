@@ -133,11 +133,12 @@ size_t route_pairs_smem(const Model &m);
 // then the serial chain.
 //   ctab: scratch of seq_table_floats(D, Qs) floats;
 //   aux: scratch of seq_aux_floats(D, M, H1, Qs) floats;
+//   more: the call has a further chunk, whose preparation comes next;
 //   slots: table blocks resident on the whole GPU at once (seq_table_slots).
 cudaError_t launch_seq_table(const Model &m, const Queries &q, int Qs, int slots,
                              float *ctab, float *aux, cudaStream_t s);
 cudaError_t launch_seq_chain(const Model &m, const Queries &q, int Qs,
-                             const float *ctab, float *aux, cudaStream_t s);
+                             const float *ctab, float *aux, bool more, cudaStream_t s);
 size_t seq_aux_floats(int D, int M, int H1, int Qs);
 // Sequential mode with the table on the tensor cores (bf16 contexts): the
 // preparation kernel alone, also writing bf16 prefixes pre_bf [D (Qs + 1)][H1]
@@ -147,7 +148,8 @@ size_t seq_aux_floats(int D, int M, int H1, int Qs);
 cudaError_t launch_seq_prep_tc(const Model &m, const Queries &q, int Qs, float *aux,
                                uint16_t *pre_bf, int32_t *dmv, cudaStream_t s);
 cudaError_t launch_seq_chain_tc(const Model &m, const Queries &q, int Qs, const float *ctab,
-                                float *aux, const float *qual, int qstride, cudaStream_t s);
+                                float *aux, const float *qual, int qstride, bool more,
+                                cudaStream_t s);
 int seq_table_slots(const Model &m);
 // Decision maker for K lambdas from stored scores: C [Q][D], quality
 // qual[q * qstride + model]; outputs [K][ostride] starting at query 0.
