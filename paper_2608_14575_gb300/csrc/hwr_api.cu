@@ -734,7 +734,11 @@ static hwr_status run_kernels(hwr_ctx *c, const Queries &q, uint32_t flags, bool
             TRY(grow(c, &c->qual, &c->qual_cap, 2 * (size_t)Qs * c->Mpad));
         }
         TRY(grow(c, &c->ctab, &c->ctab_cap, seq_table_floats(c->D, Qs)));
-        TRY(grow(c, &c->qseq, &c->qseq_cap, seq_aux_floats(c->D, c->M, c->H1, Qs)));
+        // (SIMT table: whole chunks whose prefixes are prepared at once)
+        const int run = tcs ? Qs : (SEQ_RUN / Qs > 1 ? SEQ_RUN / Qs : 1) * Qs;
+        TRY(grow(c, &c->qseq, &c->qseq_cap,
+                 seq_aux_floats(c->D, c->M, c->H1, run < q.Q ? run : q.Q)));
+        int run_lo = 0, run_n = 0;
         const size_t es = c->dtype == HWR_BF16 ? 2 : 4;
         for (int lo = 0; lo < q.Q; lo += Qs) {
             Queries k = q;
@@ -767,7 +771,7 @@ static hwr_status run_kernels(hwr_ctx *c, const Queries &q, uint32_t flags, bool
                 kt.slo_mode = 0;      // budgets are the chain's business
                 kt.slo_q = nullptr;
                 LaunchScope a(c, HWR_K_SEQ_TABLE, prof);
-                CK(c, launch_seq_prep_tc(m, k, n, c->qseq, c->prebf, c->dmv, c->stream),
+                CK(c, launch_seq_prep(m, k, n, c->qseq, c->prebf, c->dmv, c->stream),
                    "sequential preparation");
                 // fixed halves of the buffer (calls of different sizes must not
                 // overlap the half the previous call's kernels still read)
@@ -793,14 +797,24 @@ static hwr_status run_kernels(hwr_ctx *c, const Queries &q, uint32_t flags, bool
                 continue;
             }
             LaunchScope a(c, HWR_K_SEQ_TABLE, prof);
-            CK(c, launch_seq_table(m, k, n, c->seq_slots, c->ctab, c->qseq, c->stream),
+            if (lo == run_lo + run_n) {
+                run_lo = lo;
+                run_n = q.Q - lo < run ? q.Q - lo : run;
+                Queries kr = k;
+                kr.Q = run_n;
+                CK(c, launch_seq_prep(m, kr, run_n, c->qseq, nullptr, nullptr, c->stream),
+                   "sequential preparation");
+                c->stats.kernel_launches++;
+                c->stats.launches[HWR_K_SEQ_TABLE]++;
+            }
+            CK(c, launch_seq_table(m, k, n, run_n, lo - run_lo, c->seq_slots, c->ctab, c->qseq,
+                                   c->stream),
                "sequential table");
             a.done();
-            CK(c, launch_seq_chain(m, k, n, c->ctab, c->qseq, lo + Qs < q.Q, c->stream),
+            CK(c, launch_seq_chain(m, k, n, run_n, c->ctab, c->qseq, lo + Qs < q.Q, c->stream),
                "sequential chain");
-            // the preparation kernel (inside launch_seq_table) and the chain
-            c->stats.kernel_launches += 2;
-            c->stats.launches[HWR_K_SEQ_TABLE] += 2;
+            c->stats.kernel_launches++;
+            c->stats.launches[HWR_K_SEQ_TABLE]++;
         }
         return HWR_OK;
     }

@@ -17,6 +17,7 @@ constexpr int SIMT_KC = 32;          // K chunk of the layer-2 tile (64 rows: 8 
 constexpr int MAX_D = 64;
 constexpr int MAX_H = 256;
 constexpr int SEQ_MAX_CHUNK = 64;    // queries per sequential table
+constexpr int SEQ_RUN = 1024;        // queries whose prefixes are prepared at once
 constexpr int SEQ_CHAIN_SMEM = 200 * 1024;
 
 // Read-only device view of the predictor and deployment state.
@@ -127,26 +128,30 @@ constexpr int PAIRS_MAX_PAIRS = 2048;   // default upper bound on Q * D for this
 cudaError_t launch_route_pairs(const Model &m, const Queries &q, float *pairC, float *qualS,
                                float *h2, int32_t *count, int nsm, cudaStream_t s);
 size_t route_pairs_smem(const Model &m);
-// Sequential mode over one chunk of Qs <= seq_chunk(m) queries: the chunk's
-// standardised features and layer-1 prefixes, and the score table (every
-// (picks c, deployment d, query i >= c)) in launch_seq_table (two kernels),
-// then the serial chain.
+// Sequential mode.  A run of at most SEQ_RUN queries is prepared at once
+// (launch_seq_prep: Ns standardised query slots, and every deployment's layer-1
+// prefix at each count of picks it can reach); then each of its chunks of
+// Qs <= seq_chunk(m) queries, off0 queries into the run, has its score table
+// (every (picks c in the chunk, deployment d, query i >= c)) and its serial
+// chain.  q holds the run's queries for the preparation, the chunk's for the
+// other two.
 //   ctab: scratch of seq_table_floats(D, Qs) floats;
-//   aux: scratch of seq_aux_floats(D, M, H1, Qs) floats;
-//   more: the call has a further chunk, whose preparation comes next;
-//   slots: table blocks resident on the whole GPU at once (seq_table_slots).
-cudaError_t launch_seq_table(const Model &m, const Queries &q, int Qs, int slots,
+//   aux: scratch of seq_aux_floats(D, M, H1, Ns) floats;
+//   more: the call has a further chunk, which comes next;
+//   slots: table blocks resident on the whole GPU at once (seq_table_slots);
+//   pre_bf, dmv (or null): bf16 prefixes [D (Ns + 1)][H1] and the model of each
+//   (deployment, count) group d (Ns + 1) + c, for the tensor-core table.
+cudaError_t launch_seq_prep(const Model &m, const Queries &q, int Ns, float *aux, uint16_t *pre_bf,
+                            int32_t *dmv, cudaStream_t s);
+cudaError_t launch_seq_table(const Model &m, const Queries &q, int Qs, int Ns, int off0, int slots,
                              float *ctab, float *aux, cudaStream_t s);
-cudaError_t launch_seq_chain(const Model &m, const Queries &q, int Qs,
-                             const float *ctab, float *aux, bool more, cudaStream_t s);
-size_t seq_aux_floats(int D, int M, int H1, int Qs);
-// Sequential mode with the table on the tensor cores (bf16 contexts): the
-// preparation kernel alone, also writing bf16 prefixes pre_bf [D (Qs + 1)][H1]
-// and the model of each (deployment, count) group dmv [D (Qs + 1)] (group
-// d (Qs + 1) + c); the chain over the triangular table ctab (written by the
-// predictor kernel with q.seq_n = Qs) with quality rows qual [Qs][qstride].
-cudaError_t launch_seq_prep_tc(const Model &m, const Queries &q, int Qs, float *aux,
-                               uint16_t *pre_bf, int32_t *dmv, cudaStream_t s);
+cudaError_t launch_seq_chain(const Model &m, const Queries &q, int Qs, int Ns, const float *ctab,
+                             float *aux, bool more, cudaStream_t s);
+size_t seq_aux_floats(int D, int M, int H1, int Ns);
+// With the table on the tensor cores (bf16 contexts): each chunk is prepared
+// by itself (Ns = Qs), the predictor kernel writes the triangular table ctab
+// (with q.seq_n = Qs), and the chain takes its quality rows from qual
+// [Qs][qstride].
 cudaError_t launch_seq_chain_tc(const Model &m, const Queries &q, int Qs, const float *ctab,
                                 float *aux, const float *qual, int qstride, bool more,
                                 cudaStream_t s);

@@ -960,31 +960,36 @@ k_route_rows(Model m, Queries q, int32_t *status) {
 
 size_t seq_table_floats(int D, int Qs) { return tri_off(D, Qs, Qs); }
 
-// Per-chunk auxiliary arrays (one scratch buffer, seq_aux_floats floats):
-// quality [Qs][M], standardised query slots u [Qs] and v [Qs], and, for every
-// deployment d and count c = 0 .. Qs of further picks, the standardised
-// running count xr [D][Qs + 1] and the layer-1 prefix through slot F - 3
-// pre [D][Qs + 1][H1] (the snapshot kernel's chain with running r_d + c).
+// Auxiliary arrays (one scratch buffer, seq_aux_floats floats) of a run of
+// chunks, Ns queries in all: a chunk's quality [<= SEQ_MAX_CHUNK][M], the
+// queries' standardised slots u [Ns] and v [Ns], and, for every deployment d
+// and count c = 0 .. Ns of picks since the run began, the standardised running
+// count xr [D][Ns + 1] and the layer-1 prefix through slot F - 3
+// pre [D][Ns + 1][H1] (the snapshot kernel's chain with running rbase[d] + c,
+// rbase [D] the running counts as the run began).
 struct SeqAux {
-    float *qual, *us, *vs, *xr, *pre;
+    float *qual, *us, *vs, *xr;
+    int32_t *rbase;
+    float *pre;
 };
 
-__host__ __device__ inline SeqAux seq_aux(float *aux, int D, int M, int Qs) {
+__host__ __device__ inline SeqAux seq_aux(float *aux, int D, int M, int Ns) {
     SeqAux a;
     a.qual = aux;
-    a.us = aux + (size_t)Qs * M;
-    a.vs = a.us + Qs;
-    a.xr = a.vs + Qs;
-    a.pre = a.xr + (((size_t)D * (Qs + 1) + 3) & ~(size_t)3);
+    a.us = aux + (size_t)SEQ_MAX_CHUNK * M;
+    a.vs = a.us + Ns;
+    a.xr = a.vs + Ns;
+    a.rbase = reinterpret_cast<int32_t *>(a.xr + (size_t)D * (Ns + 1));
+    a.pre = aux + (((size_t)SEQ_MAX_CHUNK * M + 2 * (size_t)Ns + (size_t)D * (Ns + 2) + 3) & ~(size_t)3);
     return a;
 }
 
-size_t seq_aux_floats(int D, int M, int H1, int Qs) {
-    return (size_t)Qs * M + 2 * (size_t)Qs + (((size_t)D * (Qs + 1) + 3) & ~(size_t)3) +
-           (size_t)D * (Qs + 1) * H1;
+size_t seq_aux_floats(int D, int M, int H1, int Ns) {
+    return (((size_t)SEQ_MAX_CHUNK * M + 2 * (size_t)Ns + (size_t)D * (Ns + 2) + 3) & ~(size_t)3) +
+           (size_t)D * (Ns + 1) * H1;
 }
 
-// K_seq_prep: the chunk's standardised features and layer-1 prefixes, each
+// K_seq_prep: a run's standardised features and layer-1 prefixes, each
 // computed once (double arithmetic is scarce on this GPU, and every table
 // block would otherwise repeat it).  Blocks [0, nuv): the query slots; then
 // one block per deployment d and run of PREP_COUNTS counts c.
@@ -1027,6 +1032,7 @@ k_seq_prep(Model m, Queries q, int Qs, float *aux, uint16_t *pre_bf, int32_t *dm
                                     m.sd[P + 1]);
         xr[tid] = v;
         a.xr[g0 + tid] = v;
+        if (c0 + tid == 0) a.rbase[d] = m.running[d];
         if (dmv) dmv[g0 + tid] = m.dep_model[d];
     } else if (tid < PREP_COUNTS) {
         xr[tid] = 0.f;   // past the last count: computed, never stored
@@ -1083,7 +1089,7 @@ struct FlatRows {
 };
 
 struct SeqLayout {
-    size_t us, vs, gi, qi, sp, w3, w1q, tile, total;
+    size_t us, vs, gi, qi, di, sp, w3, w1q, tile, total;
 };
 
 __host__ __device__ inline SeqLayout seq_layout(int H2) {
@@ -1093,6 +1099,7 @@ __host__ __device__ inline SeqLayout seq_layout(int H2) {
     L.vs = o; o += SEQ_MAX_CHUNK;
     L.gi = o; o += TILE_ROWS;
     L.qi = o; o += TILE_ROWS;
+    L.di = o; o += TILE_ROWS;
     L.sp = o; o += 3 * TILE_ROWS;
     o = (o + 3) & ~(size_t)3;   // W3 rows read as 16-byte vectors
     L.w3 = o; o += 3 * (size_t)H2;
@@ -1115,23 +1122,25 @@ __host__ __device__ inline int seq_qual_rows(int M) {
 // so that every SM gets the same number of rows.
 template <int CPT>
 __global__ void __launch_bounds__(SIMT_THREADS, CPT <= 4 ? 3 : 2)
-k_seq_table(Model m, Queries q, int Qs, int nb_qual, int rows_per_block, float *ctab,
-            float *aux) {
+k_seq_table(Model m, Queries q, int Qs, int Ns, int off0, int nb_qual, int rows_per_block,
+            float *ctab, float *aux) {
     extern __shared__ float4 sm4[];
     float *sm = reinterpret_cast<float *>(sm4);
     const int tid = threadIdx.x;
     const int D = m.D, M = m.M;
     const SeqLayout L = seq_layout(m.H2);
-    const SeqAux A = seq_aux(aux, D, M, Qs);
-    // launched as a programmatic dependent of the preparation kernel: the
-    // chain may be scheduled now; the quality blocks need nothing from the
-    // preparation kernel, the table blocks wait for it below
+    const SeqAux A = seq_aux(aux, D, M, Ns);
+    // launched as a programmatic dependent of the preparation kernel, or of the
+    // chain of the chunk before: the chain may be scheduled now; nothing that
+    // those kernels write is read, and nothing they read is written, before
+    // this grid has waited for them
     umma::grid_launch_dependents();
     if ((int)blockIdx.x < nb_qual) {
         // quality of the chunk's queries [q0, q0 + nq), staged through the whole
         // shared space
         const int nq = seq_qual_rows(M), q0 = (int)blockIdx.x * nq;
         const float v = quality_staged(m, q, q0, nq, sm, (int)L.total);
+        umma::grid_dependency_wait();
         if (tid < nq * M && q0 + tid / M < Qs) A.qual[(size_t)q0 * M + tid] = v;
         return;
     }
@@ -1140,6 +1149,7 @@ k_seq_table(Model m, Queries q, int Qs, int nb_qual, int rows_per_block, float *
     const int R = min(rows_per_block, T - t0);
     float *us = sm + L.us, *vs = sm + L.vs, *sp = sm + L.sp;
     int *gi = reinterpret_cast<int *>(sm + L.gi), *qi = reinterpret_cast<int *>(sm + L.qi);
+    int *di = reinterpret_cast<int *>(sm + L.di);
     for (int r = tid; r < R; r += SIMT_THREADS) {
         // entry t: the count c with tri_off(c) <= t < tri_off(c + 1), then d and i
         const int t = t0 + r;
@@ -1150,16 +1160,20 @@ k_seq_table(Model m, Queries q, int Qs, int nb_qual, int rows_per_block, float *
             else hi = mid - 1;
         }
         const int off = t - (int)tri_off(D, Qs, lo), len = Qs - lo, d = off / len;
-        gi[r] = d * (Qs + 1) + lo;
+        gi[r] = d * (Ns + 1) + lo;
+        di[r] = d;
         qi[r] = lo + off - d * len;
     }
     // the weights need nothing from the preparation kernel
     pair_mlp_stage<CPT>(m, sm + L.tile, sm + L.w3, sm + L.w1q);
-    umma::grid_dependency_wait();    // the preparation kernel's features and prefixes
+    umma::grid_dependency_wait();    // the run's features and prefixes, the picks so far
     for (int i = tid; i < Qs; i += SIMT_THREADS) {
-        us[i] = A.us[i];
-        vs[i] = A.vs[i];
+        us[i] = A.us[off0 + i];
+        vs[i] = A.vs[off0 + i];
     }
+    // counts are of the run: the deployment's picks in the chunks before count too
+    for (int r = tid; r < R; r += SIMT_THREADS)
+        gi[r] += __ldcg(m.running + di[r]) - __ldcg(A.rbase + di[r]);
     __syncthreads();
 
     FlatRows rows{A.pre, gi, qi, m.H1};
@@ -1193,13 +1207,13 @@ __device__ __forceinline__ float warp_max(float x) {
 // fit in shared memory; the walk reads the rest from global memory (L2).
 template <bool HI, bool BIG>
 __global__ void __launch_bounds__(CHAIN_THREADS)
-k_seq_chain(Model m, Queries q, int Qs, const float *ctab, float *aux, const float *qsrc,
+k_seq_chain(Model m, Queries q, int Qs, int Ns, const float *ctab, float *aux, const float *qsrc,
             int qstride, int tsm, int more) {
     extern __shared__ float4 sm4[];
     float *sm = reinterpret_cast<float *>(sm4);
     const int tid = threadIdx.x, lane = tid & 31;
     const int D = m.D, M = m.M, F = m.F, H1 = m.H1, P = m.P;
-    const SeqAux A = seq_aux(aux, D, M, Qs);
+    const SeqAux A = seq_aux(aux, D, M, Ns);
     const size_t T = tri_off(D, Qs, Qs);
     int *dm = reinterpret_cast<int *>(sm), *cnt = dm + MAX_D, *o_ch = cnt + MAX_D;
     float *tab = sm + 2 * MAX_D + SEQ_MAX_CHUNK;
@@ -1217,10 +1231,11 @@ k_seq_chain(Model m, Queries q, int Qs, const float *ctab, float *aux, const flo
     // launched as a programmatic dependent of the table kernel: budgets and
     // the model map first, then wait for the table (and, through it, for the
     // preparation kernel)
-    // the next chunk's preparation may be launched now (it waits for this grid
-    // before it does anything); after the last chunk anything may follow, the
-    // tensor-core route among them, whose predictor reads the prefixes that
-    // this kernel persists without waiting for more than the kernel before it
+    // the call's next chunk may be launched now (its table, or the preparation
+    // of a further run of chunks: both wait for this grid before they touch
+    // what it uses); after the last chunk anything may follow, the tensor-core
+    // route among them, whose predictor reads the prefixes that this kernel
+    // persists without waiting for more than the kernel before it
     if (more) umma::grid_launch_dependents();
     for (int i = tid; i < Qs; i += CHAIN_THREADS) slo[i] = query_budget(q, i);
     for (int e = tid; e < D; e += CHAIN_THREADS) dm[e] = m.dep_model[e];
@@ -1425,16 +1440,20 @@ k_seq_chain(Model m, Queries q, int Qs, const float *ctab, float *aux, const flo
     }
     __syncthreads();
 
-    // persist the picks and refresh the state they touch: the standardised
-    // running count and the layer-1 prefix are the preparation kernel's values
-    // for the final count
-    for (int d = tid; d < D; d += CHAIN_THREADS) {
-        m.running[d] += cnt[d];
-        m.X[(size_t)d * F + P + 1] = A.xr[(size_t)d * (Qs + 1) + cnt[d]];
+    // persist the picks and, after the call's last chunk, the state they touch:
+    // the standardised running count and the layer-1 prefix are the preparation
+    // kernel's values for the final count
+    if (tid < D) {
+        const int r = m.running[tid] + cnt[tid];
+        m.running[tid] = r;
+        cnt[tid] = tid * (Ns + 1) + r - A.rbase[tid];
+        if (!more) m.X[(size_t)tid * F + P + 1] = A.xr[cnt[tid]];
     }
+    if (more) return;
+    __syncthreads();
     for (int e = tid; e < D * H1; e += CHAIN_THREADS) {
         const int d = e / H1, j = e - d * H1;
-        const float v = A.pre[((size_t)d * (Qs + 1) + cnt[d]) * H1 + j];
+        const float v = A.pre[(size_t)cnt[d] * H1 + j];
         m.A[e] = v;
         m.Abf[e] = __bfloat16_as_ushort(__float2bfloat16_rn(v));
     }
@@ -2315,10 +2334,8 @@ cudaError_t launch_select_multi(const Model &m, const Queries &q, const float *C
     return cudaGetLastError();
 }
 
-cudaError_t launch_seq_table(const Model &m, const Queries &q, int Qs, int slots, float *ctab,
-                             float *aux, cudaStream_t s) {
-    cudaError_t e = launch_seq_prep_tc(m, q, Qs, aux, nullptr, nullptr, s);
-    if (e != cudaSuccess) return e;
+cudaError_t launch_seq_table(const Model &m, const Queries &q, int Qs, int Ns, int off0, int slots,
+                             float *ctab, float *aux, cudaStream_t s) {
     // rows per table block: a multiple of 8 (whole warps of the tile) that
     // spreads the table evenly over the blocks resident at once
     const int T = (int)tri_off(m.D, Qs, Qs);
@@ -2329,10 +2346,10 @@ cudaError_t launch_seq_table(const Model &m, const Queries &q, int Qs, int slots
     const int blocks = nb_qual + (T + rpb - 1) / rpb;
     cudaLaunchConfig_t cfg = dependent_launch(blocks, SIMT_THREADS, seq_layout(m.H2).total * sizeof(float), s);
     switch (cpt_for(m.H2)) {
-        case 1: return cudaLaunchKernelEx(&cfg, k_seq_table<1>, m, q, Qs, nb_qual, rpb, ctab, aux);
-        case 2: return cudaLaunchKernelEx(&cfg, k_seq_table<2>, m, q, Qs, nb_qual, rpb, ctab, aux);
-        case 4: return cudaLaunchKernelEx(&cfg, k_seq_table<4>, m, q, Qs, nb_qual, rpb, ctab, aux);
-        default: return cudaLaunchKernelEx(&cfg, k_seq_table<8>, m, q, Qs, nb_qual, rpb, ctab, aux);
+        case 1: return cudaLaunchKernelEx(&cfg, k_seq_table<1>, m, q, Qs, Ns, off0, nb_qual, rpb, ctab, aux);
+        case 2: return cudaLaunchKernelEx(&cfg, k_seq_table<2>, m, q, Qs, Ns, off0, nb_qual, rpb, ctab, aux);
+        case 4: return cudaLaunchKernelEx(&cfg, k_seq_table<4>, m, q, Qs, Ns, off0, nb_qual, rpb, ctab, aux);
+        default: return cudaLaunchKernelEx(&cfg, k_seq_table<8>, m, q, Qs, Ns, off0, nb_qual, rpb, ctab, aux);
     }
 }
 
@@ -2353,23 +2370,23 @@ int seq_table_slots(const Model &m) {
     return nsm * per;
 }
 
-cudaError_t launch_seq_chain(const Model &m, const Queries &q, int Qs, const float *ctab,
+cudaError_t launch_seq_chain(const Model &m, const Queries &q, int Qs, int Ns, const float *ctab,
                              float *aux, bool more, cudaStream_t s) {
     cudaLaunchConfig_t cfg = dependent_launch(1, CHAIN_THREADS, chain_smem(m.D, m.M, Qs), s);
-    const SeqAux A = seq_aux(aux, m.D, m.M, Qs);
+    const SeqAux A = seq_aux(aux, m.D, m.M, Ns);
     if (m.D > 32)
-        return cudaLaunchKernelEx(&cfg, k_seq_chain<true, false>, m, q, Qs, ctab, aux,
+        return cudaLaunchKernelEx(&cfg, k_seq_chain<true, false>, m, q, Qs, Ns, ctab, aux,
                                   (const float *)A.qual, m.M, 0, (int)more);
-    return cudaLaunchKernelEx(&cfg, k_seq_chain<false, false>, m, q, Qs, ctab, aux,
+    return cudaLaunchKernelEx(&cfg, k_seq_chain<false, false>, m, q, Qs, Ns, ctab, aux,
                               (const float *)A.qual, m.M, 0, (int)more);
 }
 
-cudaError_t launch_seq_prep_tc(const Model &m, const Queries &q, int Qs, float *aux,
-                               uint16_t *pre_bf, int32_t *dmv, cudaStream_t s) {
-    const int nuv = (2 * Qs + PREP_THREADS - 1) / PREP_THREADS;
+cudaError_t launch_seq_prep(const Model &m, const Queries &q, int Ns, float *aux, uint16_t *pre_bf,
+                            int32_t *dmv, cudaStream_t s) {
+    const int nuv = (2 * Ns + PREP_THREADS - 1) / PREP_THREADS;
     cudaLaunchConfig_t cfg =
-        dependent_launch(nuv + m.D * seq_prep_blocks_per_dep(Qs), PREP_THREADS, 0, s);
-    return cudaLaunchKernelEx(&cfg, k_seq_prep, m, q, Qs, aux, pre_bf, dmv);
+        dependent_launch(nuv + m.D * seq_prep_blocks_per_dep(Ns), PREP_THREADS, 0, s);
+    return cudaLaunchKernelEx(&cfg, k_seq_prep, m, q, Ns, aux, pre_bf, dmv);
 }
 
 cudaError_t launch_seq_chain_tc(const Model &m, const Queries &q, int Qs, const float *ctab,
@@ -2378,9 +2395,9 @@ cudaError_t launch_seq_chain_tc(const Model &m, const Queries &q, int Qs, const 
     if (chain_smem(m.D, m.M, Qs) <= (size_t)SEQ_CHAIN_SMEM) {
         cudaLaunchConfig_t cfg = dependent_launch(1, CHAIN_THREADS, chain_smem(m.D, m.M, Qs), s);
         if (m.D > 32)
-            return cudaLaunchKernelEx(&cfg, k_seq_chain<true, false>, m, q, Qs, ctab, aux, qual,
+            return cudaLaunchKernelEx(&cfg, k_seq_chain<true, false>, m, q, Qs, Qs, ctab, aux, qual,
                                       qstride, 0, (int)more);
-        return cudaLaunchKernelEx(&cfg, k_seq_chain<false, false>, m, q, Qs, ctab, aux, qual,
+        return cudaLaunchKernelEx(&cfg, k_seq_chain<false, false>, m, q, Qs, Qs, ctab, aux, qual,
                                   qstride, 0, (int)more);
     }
     // the table's first rows in shared memory, the rest read from L2
@@ -2390,9 +2407,9 @@ cudaError_t launch_seq_chain_tc(const Model &m, const Queries &q, int Qs, const 
     cudaLaunchConfig_t cfg =
         dependent_launch(1, CHAIN_THREADS, rest + (size_t)tsm * sizeof(float), s);
     if (m.D > 32)
-        return cudaLaunchKernelEx(&cfg, k_seq_chain<true, true>, m, q, Qs, ctab, aux, qual,
+        return cudaLaunchKernelEx(&cfg, k_seq_chain<true, true>, m, q, Qs, Qs, ctab, aux, qual,
                                   qstride, tsm, (int)more);
-    return cudaLaunchKernelEx(&cfg, k_seq_chain<false, true>, m, q, Qs, ctab, aux, qual, qstride,
+    return cudaLaunchKernelEx(&cfg, k_seq_chain<false, true>, m, q, Qs, Qs, ctab, aux, qual, qstride,
                               tsm, (int)more);
 }
 

@@ -66,3 +66,30 @@ def test_values_off_the_ordinary_range(M, G, what, slo):
         p["W1"] = np.zeros_like(p["W1"])
         p["memb"] = np.zeros_like(p["memb"])
     _check(p)
+
+
+@pytest.mark.parametrize("M,G,Q", [(4, 3, 1024), (5, 1, 1025), (4, 3, 2100), (16, 4, 1200)])
+def test_runs_of_chunks(M, G, Q):
+    """Calls longer than one run of prepared prefixes, and a second call that
+    continues from the first one's counts."""
+    p = _problem(Q, M, G)
+    p["slo"] = 4.0
+    _check(p)
+    r = H.Router(p)
+    orc = O.Problem(p)
+    running = p["snap"]["running"]
+    for lo, hi in ((0, 130), (130, Q)):
+        s = W.query_slice(p, lo, hi)
+        got = r.route(s["in_len"], s["out_len"], s["emb"], flags=H.HWR_SEQUENTIAL)
+        want = orc.route(s["in_len"], s["out_len"], s["emb"], mode=O.F32, sequential=True, running=running)
+        for g, w, t in zip(got, want, (np.int32, np.float32, np.float32)):
+            assert np.array_equal(g, np.asarray(w).astype(t), equal_nan=True)
+        running = want[3]
+        assert np.array_equal(r.get_snapshot(), running)
+    # a batch route after it sees the prefixes of the final counts
+    got = r.route(p["in_len"][:50], p["out_len"][:50], p["emb"][:50], flags=H.HWR_PATH_SIMT)
+    snap = dict(p["snap"], running=running)
+    orc.set_snapshot(snap)
+    want = orc.route(p["in_len"][:50], p["out_len"][:50], p["emb"][:50], mode=O.F32)
+    assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1].astype(np.float32))
+    r.close()
