@@ -2334,17 +2334,60 @@ cudaError_t launch_select_multi(const Model &m, const Queries &q, const float *C
     return cudaGetLastError();
 }
 
+// Blocks of a chunk's table: quality blocks, and blocks of rpb rows (a multiple
+// of 8, whole warps of the tile) that spread the table evenly over the blocks
+// resident at once.
+struct SeqGrid {
+    int nb_qual, rpb, blocks;
+};
+
+static SeqGrid seq_grid(const Model &m, int Qs, int slots) {
+    SeqGrid g;
+    const int T = (int)tri_off(m.D, Qs, Qs);
+    g.nb_qual = (Qs + seq_qual_rows(m.M) - 1) / seq_qual_rows(m.M);
+    const int want = slots - g.nb_qual > 1 ? slots - g.nb_qual : 1;
+    const int rpb = ((T + want - 1) / want + 7) / 8 * 8;
+    g.rpb = rpb < 8 ? 8 : (rpb > TILE_ROWS ? TILE_ROWS : rpb);
+    g.blocks = g.nb_qual + (T + g.rpb - 1) / g.rpb;
+    return g;
+}
+
+// Queries per chunk of a sequential call of Q.  A chunk costs a fixed part (its
+// launches, the tables' serial parts, the walk and its copy) and its table's
+// rounds of blocks of rpb rows; the table grows with the square of a chunk, so
+// wide clusters take shorter chunks.  Both parts grow with H1; the constants
+// fit chunks of 8 to 64 queries measured on GB300 (us: H = 64, D = 32: 9.8 and
+// 0.14 a row; H = 128, D = 12: 13.5 and 0.38; H = 256, D = 32: 20 and 0.85;
+// shorter blocks than 24 rows wait on latencies and take as long).
+// 1,000 requests in the largest chunks that the chain takes / in the ones
+// chosen here (us): D = 12, H = 128 548 / 526; D = 32, H = 64 494 / 456;
+// D = 32, H = 256 2,689 / 1,737; D = 64, H = 256 4,432 / 3,032.
+int seq_pick_chunk(const Model &m, int Q, int limit, int slots) {
+    const double fixed_us = 6.4 + 0.053 * m.H1;
+    const double row_us = m.H1 > 21 ? 0.0033 * m.H1 - 0.04 : 0.03;
+    int best = limit;
+    double best_cost = 1e300;
+    for (int n = (Q + limit - 1) / limit;; ++n) {
+        const int Qs = (Q + n - 1) / n;
+        const SeqGrid g = seq_grid(m, Qs, slots);
+        const double rounds = g.blocks > slots ? (double)g.blocks / slots : 1.0;
+        const double cost = ((Q + Qs - 1) / Qs) * (fixed_us + row_us * (g.rpb > 24 ? g.rpb : 24) * rounds);
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = Qs;
+        }
+        if (Qs <= 8) break;
+        // the next chunk size below this one
+        n = (Q + Qs - 2) / (Qs - 1) - 1 > n ? (Q + Qs - 2) / (Qs - 1) - 1 : n;
+    }
+    return best;
+}
+
 cudaError_t launch_seq_table(const Model &m, const Queries &q, int Qs, int Ns, int off0, int slots,
                              float *ctab, float *aux, cudaStream_t s) {
-    // rows per table block: a multiple of 8 (whole warps of the tile) that
-    // spreads the table evenly over the blocks resident at once
-    const int T = (int)tri_off(m.D, Qs, Qs);
-    const int nb_qual = (Qs + seq_qual_rows(m.M) - 1) / seq_qual_rows(m.M);
-    const int want = slots - nb_qual > 1 ? slots - nb_qual : 1;
-    int rpb = ((T + want - 1) / want + 7) / 8 * 8;
-    rpb = rpb < 8 ? 8 : (rpb > TILE_ROWS ? TILE_ROWS : rpb);
-    const int blocks = nb_qual + (T + rpb - 1) / rpb;
-    cudaLaunchConfig_t cfg = dependent_launch(blocks, SIMT_THREADS, seq_layout(m.H2).total * sizeof(float), s);
+    const SeqGrid g = seq_grid(m, Qs, slots);
+    const int nb_qual = g.nb_qual, rpb = g.rpb;
+    cudaLaunchConfig_t cfg = dependent_launch(g.blocks, SIMT_THREADS, seq_layout(m.H2).total * sizeof(float), s);
     switch (cpt_for(m.H2)) {
         case 1: return cudaLaunchKernelEx(&cfg, k_seq_table<1>, m, q, Qs, Ns, off0, nb_qual, rpb, ctab, aux);
         case 2: return cudaLaunchKernelEx(&cfg, k_seq_table<2>, m, q, Qs, Ns, off0, nb_qual, rpb, ctab, aux);
