@@ -192,7 +192,9 @@ hwr_status hwr_get_snapshot(hwr_ctx *ctx, int32_t *running_out);
  * there, so the arrays must stay untouched until the call returns.  Pinned
  * host memory gives the full
  * link bandwidth.  With HWR_DEVICE_PTRS they are device pointers read and
- * written in stream order.  With HWR_ASYNC the call returns after enqueueing;
+ * written in stream order; without HWR_ASYNC such a call, too, returns as soon
+ * as every output is written (and every input read), possibly before the
+ * kernel's last blocks retire.  With HWR_ASYNC the call returns after enqueueing;
  * host arrays must then stay valid until hwr_synchronize().
  * HWR_SEQUENTIAL: queries are routed in index order and each decision
  * increments its deployment's running count before the next query is scored;

@@ -121,6 +121,14 @@ struct hwr_ctx {
     // the most recent predictor launch
     uint32_t *done_d = nullptr;
     uint32_t pred_ctas = 0, pred_ctas_last = 0;
+    // waited device calls: a mapped host word that the call's last block sets
+    // (HostFlag), the fused kernel's block counter (device) and the blocks
+    // counted on it, the word's value for the call that waits
+    int32_t *flag_h = nullptr, *flag_d = nullptr;
+    uint32_t *simt_done_d = nullptr;
+    uint32_t simt_blocks = 0;
+    int32_t flag_seq = 0;
+    bool want_flag = false, flagged = false;    // this call wants one; its kernel sets one
     // outputs of the last tensor-core route (its predictor may still run
     // while the next route's kernels start)
     struct Range {
@@ -507,6 +515,8 @@ static hwr_status build_ctx(hwr_ctx *c, const hwr_deployment_table *t, const hwr
         for (int k = 0; k < F; ++k) w1t[(size_t)k * H1 + j] = w1[(size_t)j * F + k];
     TRY(upload(c, c->W1T, w1t.data(), w1t.size() * 4, "upload W1 transposed"));
     CK(c, cudaMemset(c->pairN, 0, 2 * PAIRS_MAX_PAIRS * sizeof(int32_t)), "zero counters");
+    TRY(dev_alloc(c, &c->simt_done_d, 1));
+    CK(c, cudaMemset(c->simt_done_d, 0, sizeof(uint32_t)), "zero block counter");
     c->xform_h.assign(p->feat_xform, p->feat_xform + F);
     c->mu_in = p->feat_mean[F - 2]; c->sd_in = p->feat_std[F - 2]; c->xf_in = p->feat_xform[F - 2];
     c->mu_out = p->feat_mean[F - 1]; c->sd_out = p->feat_std[F - 1]; c->xf_out = p->feat_xform[F - 1];
@@ -543,6 +553,8 @@ static hwr_status build_ctx(hwr_ctx *c, const hwr_deployment_table *t, const hwr
     CK(c, cudaHostAlloc((void **)&c->status_h, 64, cudaHostAllocMapped), "alloc status word");
     memset(c->status_h, 0, 64);
     CK(c, cudaHostGetDevicePointer((void **)&c->status_d, c->status_h, 0), "map status word");
+    c->flag_h = c->status_h + 8;      // (a 32-byte sector of its own)
+    c->flag_d = c->status_d + 8;
 
     // snapshot staging: 6 arrays of D 4-byte values
     if (hook_fires(c)) return fail(c, HWR_ERR_OOM, "allocation %ld failed (test hook)", c->hook.count);
@@ -860,8 +872,15 @@ static hwr_status run_kernels(hwr_ctx *c, const Queries &q, uint32_t flags, bool
         c->prev_out[4] = {q.qual_out, q.qual_out ? qb4 * c->M : 0};
         LaunchScope b(c, HWR_K_MLP_TC, prof);
         int ctas = 0;
+        HostFlag flag;
+        if (c->want_flag) {
+            flag.word = c->flag_d;
+            flag.value = c->flag_seq;
+            flag.target = c->pred_ctas;
+            c->flagged = true;
+        }
         CK(c, launch_mlp_tc(t, q, qb, sp, c->part, c->count, c->status_d, c->stream, c->done_d,
-                            &ctas),
+                            &ctas, flag),
            "predictor kernel");
         c->pred_ctas += (uint32_t)ctas;
         c->pred_ctas_last = (uint32_t)ctas;
@@ -873,7 +892,16 @@ static hwr_status run_kernels(hwr_ctx *c, const Queries &q, uint32_t flags, bool
         CK(c, launch_route_pairs(m, q, c->pairC, c->pairQ, c->pairH, c->pairN, c->nsm, c->stream),
            "route kernel");
     else
-        CK(c, launch_route_simt(m, q, c->nsm, c->status_d, c->stream), "route kernel");
+    {
+        HostFlag flag;
+        if (c->want_flag) {
+            flag.word = c->flag_d;
+            flag.count = c->simt_done_d;
+            flag.value = c->flag_seq;
+        }
+        CK(c, launch_route_simt(m, q, c->nsm, c->status_d, flag, &c->simt_blocks, &c->flagged,
+                                c->stream), "route kernel");
+    }
     a.done();
     return HWR_OK;
 }
@@ -894,6 +922,16 @@ static bool wait_chosen(const int32_t *ch, int Q, long limit_us) {
         while (__atomic_load_n(ch + i, __ATOMIC_ACQUIRE) == OUT_PENDING)
             if ((++n & 1023u) == 0 && std::chrono::steady_clock::now() - t0 > limit) return false;
     }
+    return true;
+}
+
+// The host word of a waited device call; false after limit_us.
+static bool wait_flag(const int32_t *word, int32_t value, long limit_us) {
+    const auto t0 = std::chrono::steady_clock::now();
+    const auto limit = std::chrono::microseconds(limit_us);
+    unsigned n = 0;
+    while (__atomic_load_n(word, __ATOMIC_ACQUIRE) != value)
+        if ((++n & 1023u) == 0 && std::chrono::steady_clock::now() - t0 > limit) return false;
     return true;
 }
 
@@ -1064,6 +1102,16 @@ static hwr_status route_impl(hwr_ctx *c, int32_t Q, const float *in_len, const f
         q.util = (float *)(ob + o_util);
     }
 
+    // A waited route on device pointers: its kernel's last block sets a host
+    // word, and the host waits for that instead of synchronising the stream
+    // (256 fp32 queries at D = 4: 20.5 -> 19.2 us; 4,096 bf16 ones at D = 12:
+    // 28.3 -> 27.6)
+    c->want_flag = dev && !seq && !ml && !so && !(flags & (HWR_ASYNC | HWR_PROFILE)) && c->poll_us > 0;
+    c->flagged = false;
+    if (c->want_flag) {
+        c->flag_seq = c->flag_seq == INT32_MAX ? 1 : c->flag_seq + 1;
+        __atomic_store_n(c->flag_h, 0, __ATOMIC_RELAXED);
+    }
     const Model mv = model_view(c);
     // Stored scores: cost [Q][D] and quality [Q][M], for the selection over
     // several lambdas or as the output of hwr_score_batch.
@@ -1192,7 +1240,8 @@ static hwr_status route_impl(hwr_ctx *c, int32_t Q, const float *in_len, const f
         c->async_pending = true;
         return HWR_OK;
     }
-    if (!synced) CK(c, cudaStreamSynchronize(c->stream), "synchronize");
+    if (!synced && !(c->flagged && wait_flag(c->flag_h, c->flag_seq, c->poll_us)))
+        CK(c, cudaStreamSynchronize(c->stream), "synchronize");
     // this call's work is complete, and with it every earlier kernel
     c->async_pending = false;
     c->snap_busy = false;

@@ -109,6 +109,28 @@ __device__ __forceinline__ float query_budget(const Queries &q, int row) {
 }
 #endif
 
+// How a kernel tells a waiting host that the call's outputs are written: every
+// block counts itself on `count` as it ends, and the one that makes it `target`
+// (modulo 2^32) stores `value` in the mapped host word `word` (null: nobody waits).
+struct HostFlag {
+    int32_t *word = nullptr;
+    uint32_t *count = nullptr;
+    uint32_t target = 0;
+    int32_t value = 0;
+};
+
+#ifdef __CUDACC__
+// One thread, after the block's last access to global memory and a block
+// barrier.  The count acquires the other blocks' writes and the store releases
+// them at system scope: later work on any stream sees the outputs.
+__device__ __forceinline__ void flag_block_done(const HostFlag &f) {
+    uint32_t old;
+    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(old) : "l"(f.count) : "memory");
+    if (f.word && old + 1u == f.target)
+        asm volatile("st.release.sys.global.b32 [%0], %1;" ::"l"(f.word), "r"(f.value) : "memory");
+}
+#endif
+
 // ---- SIMT kernels (k_simt.cu) -------------------------------------------
 // The snapshot signals are read from `stage` ([6][D] 4-byte values in host
 // memory mapped into the device's address space, in the order running,
@@ -116,9 +138,11 @@ __device__ __forceinline__ float query_budget(const Queries &q, int row) {
 // starts (they are contiguous, in that order).
 cudaError_t launch_snapshot(const Model &m, const uint32_t *stage, cudaStream_t s);
 // Fused gather -> MLP -> mask -> argmax for a batch, on nsm SMs.  status: the
-// device status word (bounded waits).
+// device status word (bounded waits).  flag (its count and target are filled
+// from `blocks`, a running count of the blocks launched on the counter): the host
+// word to set at the end; *flagged: whether the kernel chosen does.
 cudaError_t launch_route_simt(const Model &m, const Queries &q, int nsm, int32_t *status,
-                              cudaStream_t s);
+                              HostFlag flag, uint32_t *blocks, bool *flagged, cudaStream_t s);
 // Small-batch (latency) variant: groups of (query, deployment) pairs with
 // layer 2 split by columns over several blocks, plus quality blocks; scratch
 // pairC [Q][D], qualS [Q][M], h2 [Q D][H2], count [2 PAIRS_MAX_PAIRS] (query
@@ -217,10 +241,12 @@ MlpSplit tc_mlp_split(const TcModel &m, int Q, int max_split = 8);
 // SMs the predictor kernel for Q queries split as sp leaves free (0 if none).
 int tc_mlp_free_sms(int Q, const MlpSplit &sp);
 // done: completion counter every CTA increments (release) as it finishes
-// (nullptr: none); *ctas: the CTAs launched (0 on failure).
+// (nullptr: none); *ctas: the CTAs launched (0 on failure); flag: host word to
+// set at the end (its count is `done`, its target the count before this launch).
 cudaError_t launch_mlp_tc(const TcModel &m, const Queries &q, const float *qual,
                           const MlpSplit &sp, void *part, int32_t *count, int32_t *status,
-                          cudaStream_t s, uint32_t *done, int *ctas);
+                          cudaStream_t s, uint32_t *done, int *ctas,
+                          HostFlag flag = HostFlag());
 cudaError_t tc_prepare();
 // Costs of every (query, deployment) pair of at most 128 queries into
 // q.pair_C [Q][m.D] (q.no_select set), the deployments spread over the SMs.

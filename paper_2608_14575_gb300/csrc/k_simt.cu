@@ -470,7 +470,8 @@ __host__ __device__ inline RouteLayout route_layout(int D, int M, int H2) {
 constexpr int ROUTE_THREADS = SIMT_THREADS + 32;
 
 template <int CPT>
-__global__ void __launch_bounds__(ROUTE_THREADS, CPT <= 4 ? 3 : 2) k_route_simt(Model m, Queries q) {
+__global__ void __launch_bounds__(ROUTE_THREADS, CPT <= 4 ? 3 : 2)
+k_route_simt(Model m, Queries q, HostFlag flag) {
     extern __shared__ float4 sm4[];
     float *sm = reinterpret_cast<float *>(sm4);
     const RouteLayout L = route_layout(m.D, m.M, m.H2);
@@ -536,6 +537,10 @@ __global__ void __launch_bounds__(ROUTE_THREADS, CPT <= 4 ? 3 : 2) k_route_simt(
             q.lat[qq] = ok ? best.C : __int_as_float(0x7fc00000);
             q.util[qq] = ok ? best.U : __int_as_float(0x7fc00000);
         }
+    }
+    if (flag.word) {
+        __syncthreads();
+        if (tid == 0) flag_block_done(flag);
     }
 }
 
@@ -2255,7 +2260,8 @@ static bool rows_kernel(const Model &m, int Q, int nsm) {
 }
 
 cudaError_t launch_route_simt(const Model &m, const Queries &q, int nsm, int32_t *status,
-                              cudaStream_t s) {
+                              HostFlag flag, uint32_t *blocks_done, bool *flagged, cudaStream_t s) {
+    *flagged = false;
     if (q.Q <= 0) return cudaSuccess;
     if (rows_kernel(m, q.Q, nsm)) {
         switch (tile_width(m.H2)) {
@@ -2268,11 +2274,16 @@ cudaError_t launch_route_simt(const Model &m, const Queries &q, int nsm, int32_t
     const RouteLayout L = route_layout(m.D, m.M, m.H2);
     const int blocks = (q.Q + L.QB - 1) / L.QB;
     const size_t smem = L.total * sizeof(float);
+    if (flag.word) {
+        *blocks_done += (uint32_t)blocks;
+        flag.target = *blocks_done;
+        *flagged = true;
+    }
     switch (cpt_for(m.H2)) {
-        case 1: k_route_simt<1><<<blocks, ROUTE_THREADS, smem, s>>>(m, q); break;
-        case 2: k_route_simt<2><<<blocks, ROUTE_THREADS, smem, s>>>(m, q); break;
-        case 4: k_route_simt<4><<<blocks, ROUTE_THREADS, smem, s>>>(m, q); break;
-        default: k_route_simt<8><<<blocks, ROUTE_THREADS, smem, s>>>(m, q); break;
+        case 1: k_route_simt<1><<<blocks, ROUTE_THREADS, smem, s>>>(m, q, flag); break;
+        case 2: k_route_simt<2><<<blocks, ROUTE_THREADS, smem, s>>>(m, q, flag); break;
+        case 4: k_route_simt<4><<<blocks, ROUTE_THREADS, smem, s>>>(m, q, flag); break;
+        default: k_route_simt<8><<<blocks, ROUTE_THREADS, smem, s>>>(m, q, flag); break;
     }
     return cudaGetLastError();
 }

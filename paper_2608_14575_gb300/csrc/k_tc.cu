@@ -450,7 +450,7 @@ template <int H2T, int NH>
 __global__ void __launch_bounds__(MLP_THREADS, 1)
 k_mlp_tc(TcModel m, Queries q, const __grid_constant__ HeadConsts hc,
          const float *__restrict__ qual, int nwhole, int nsplit, int4 *part, int32_t *count,
-         int32_t *status, uint32_t *done) {
+         int32_t *status, uint32_t *done, HostFlag flag) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *sm = align1024(smem_raw);
     constexpr bool FIXED = H2T > 0;
@@ -861,7 +861,10 @@ k_mlp_tc(TcModel m, Queries q, const __grid_constant__ HeadConsts hc,
     __syncthreads();
     // every global access of this CTA is done: count it for the quality kernel
     // that will next overwrite the quality buffer this grid read
-    if (done && tid == 0) count_release(done);
+    if (done && tid == 0) {
+        if (flag.word) flag_block_done(flag);
+        else count_release(done);
+    }
     if (warp == 0) {
         __syncwarp();
         tc_fence_after();
@@ -1005,7 +1008,7 @@ int tc_mlp_free_sms(int Q, const MlpSplit &sp) {
 
 cudaError_t launch_mlp_tc(const TcModel &m, const Queries &q, const float *qual,
                           const MlpSplit &sp, void *part, int32_t *count, int32_t *status,
-                          cudaStream_t s, uint32_t *done, int *ctas) {
+                          cudaStream_t s, uint32_t *done, int *ctas, HostFlag flag) {
     *ctas = 0;
     if (q.Q <= 0) return cudaSuccess;
     const int ntiles = (q.Q + BM - 1) / BM;
@@ -1015,6 +1018,9 @@ cudaError_t launch_mlp_tc(const TcModel &m, const Queries &q, const float *qual,
     const MlpLayout L = mlp_layout(m.H1, m.H2, m.Mpad, m.D, !mlp_fixed_h2(m.H2));
     const HeadConsts &hc = *m.head;
     int4 *pt = (int4 *)part;
+    if (!done) flag.word = nullptr;
+    flag.count = done;
+    flag.target += (uint32_t)grid;
     // programmatic dependent launch: the grid may start while the quality
     // kernel before it on the stream finishes (its epilogue waits for it)
     cudaLaunchConfig_t cfg = {};
@@ -1030,7 +1036,7 @@ cudaError_t launch_mlp_tc(const TcModel &m, const Queries &q, const float *qual,
     cudaError_t e;
 #define HWR_MLP(H2T, NHT) \
     e = cudaLaunchKernelEx(&cfg, k_mlp_tc<H2T, NHT>, m, q, hc, qual, sp.nwhole, sp.nsplit, pt, \
-                           count, status, done)
+                           count, status, done, flag)
     if (m.NH == 3) {
         if (m.H2 == 256) HWR_MLP(256, 3);
         else if (m.H2 == 128) HWR_MLP(128, 3);
