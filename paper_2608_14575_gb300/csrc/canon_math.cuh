@@ -11,8 +11,8 @@
 // good to about 2^-41, and rounded to float with Ziv's test: if adding and
 // subtracting a bound on its error rounds to the same float, that float is the
 // rounding of the exact value, and of the double-precision evaluation too
-// (whose own error is 2^-51).  Otherwise, about once in 2^14.5 values (2,882 of
-// 2^26 softplus arguments), and for arguments outside the ranges below, the
+// (whose own error is 2^-51).  Otherwise, about once in 2^15 softplus values
+// (1,451 of 2^26), and for arguments outside the ranges below, the
 // double-precision evaluation runs.  The result is the same float for every
 // argument (checked for all 2^32 of them by the tests).
 //
@@ -163,9 +163,9 @@ static __device__ __noinline__ float sigmoid_dp(float s) {
 
 // ---- canonical functions -------------------------------------------------------
 
-// Relative error bound of the two-float values.  Largest errors seen over 2^26
+// Relative error bounds of the two-float values.  Largest errors seen over 2^26
 // arguments in [-12, 12]: exp and softplus 2^-41.1, log 2^-44.1.
-constexpr float FF_ERR = 0x1p-39f;
+constexpr float FF_ERR = 0x1p-40f, FF_LOG_ERR = 0x1p-42f;
 
 // (t(raw) - mu) / sd with the slot transform t: 0 identity, 1 log1p, 2 log.
 // raw = rh + rl exactly (rl is non-zero for integers past 2^24 only).
@@ -182,7 +182,7 @@ __device__ __forceinline__ float standardise(uint8_t code, ff raw, float mu, flo
         }
         ok = ok && w.h >= 0x1p-40f && w.h <= 0x1p40f;
         t = ff_log(w);
-        err = FF_ERR * fabsf(t.h) + 0x1p-46f;
+        err = FF_LOG_ERR * fabsf(t.h) + 0x1p-48f;
     }
     const ff d = two_sum(t.h, -mu);
     const float rc = rcp_approx(sd), q = d.h * rc;
@@ -194,7 +194,7 @@ __device__ __forceinline__ float standardise(uint8_t code, ff raw, float mu, flo
     // (it is computed in single)
     ok = ok && fabsf(q) >= 0x1p-40f && fabsf(q) <= 0x1p60f && fabsf(x.l) <= 0x1p-20f * fabsf(q);
     float r;
-    if (ok && ff_round(x, err * fabsf(rc) + 0x1p-41f * fabsf(q), &r)) return r;
+    if (ok && ff_round(x, err * fabsf(rc) + 0x1p-42f * fabsf(q), &r)) return r;
     return standardise_dp(code, raw.h, raw.l, mu, sd);
 }
 

@@ -472,7 +472,9 @@ static hwr_status build_ctx(hwr_ctx *c, const hwr_deployment_table *t, const hwr
     TRY(dev_alloc(c, &c->W1T, (size_t)F * H1));
     TRY(dev_alloc(c, &c->pairC, (size_t)PAIRS_MAX_PAIRS));
     TRY(dev_alloc(c, &c->pairQ, (size_t)PAIRS_MAX_PAIRS * M));
-    TRY(dev_alloc(c, &c->pairN, 2 * (size_t)PAIRS_MAX_PAIRS));
+    // arrival counters of the small-batch kernel, and the fused kernel's block counter
+    TRY(dev_alloc(c, &c->pairN, 2 * (size_t)PAIRS_MAX_PAIRS + 1));
+    c->simt_done_d = (uint32_t *)(c->pairN + 2 * PAIRS_MAX_PAIRS);
     TRY(dev_alloc(c, &c->pairH, (size_t)PAIRS_MAX_PAIRS * H2));
     // the six snapshot arrays, contiguous: an upload lands in them directly
     TRY(dev_alloc(c, (char **)&c->snap_d, 6 * (size_t)D * 4));
@@ -514,9 +516,7 @@ static hwr_status build_ctx(hwr_ctx *c, const hwr_deployment_table *t, const hwr
     for (int j = 0; j < H1; ++j)
         for (int k = 0; k < F; ++k) w1t[(size_t)k * H1 + j] = w1[(size_t)j * F + k];
     TRY(upload(c, c->W1T, w1t.data(), w1t.size() * 4, "upload W1 transposed"));
-    CK(c, cudaMemset(c->pairN, 0, 2 * PAIRS_MAX_PAIRS * sizeof(int32_t)), "zero counters");
-    TRY(dev_alloc(c, &c->simt_done_d, 1));
-    CK(c, cudaMemset(c->simt_done_d, 0, sizeof(uint32_t)), "zero block counter");
+    CK(c, cudaMemset(c->pairN, 0, (2 * PAIRS_MAX_PAIRS + 1) * sizeof(int32_t)), "zero counters");
     c->xform_h.assign(p->feat_xform, p->feat_xform + F);
     c->mu_in = p->feat_mean[F - 2]; c->sd_in = p->feat_std[F - 2]; c->xf_in = p->feat_xform[F - 2];
     c->mu_out = p->feat_mean[F - 1]; c->sd_out = p->feat_std[F - 1]; c->xf_out = p->feat_xform[F - 1];
