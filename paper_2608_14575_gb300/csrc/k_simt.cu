@@ -482,7 +482,7 @@ k_route_simt(Model m, Queries q, HostFlag flag) {
     float *sp = sm + L.sp, *Cs = sm + L.C, *Us = sm + L.U;
 
     if (warp < SIMT_THREADS / 32) {
-        // the two query slots on two warps (their fp64 chains run side by side)
+        // the two query slots on two warps, side by side
         if (tid < QB) {
             const int qq = q0 + tid;
             us[tid] = qq < q.Q ? standardise(m.xform[F - 2], q.in_len[qq], m.mu[F - 2],
@@ -995,8 +995,7 @@ size_t seq_aux_floats(int D, int M, int H1, int Ns) {
 }
 
 // K_seq_prep: a run's standardised features and layer-1 prefixes, each
-// computed once (double arithmetic is scarce on this GPU, and every table
-// block would otherwise repeat it).  Blocks [0, nuv): the query slots; then
+// computed once (every table block would otherwise repeat it).  Blocks [0, nuv): the query slots; then
 // one block per deployment d and run of PREP_COUNTS counts c.
 constexpr int PREP_THREADS = 128;
 constexpr int PREP_COUNTS = 8;   // counts c per preparation block
@@ -1684,7 +1683,7 @@ __device__ __forceinline__ void pair_cols_split(const Model &m, const Queries &q
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     }
-    // the query slots of the group's queries (fp64 chains side by side)
+    // the query slots of the group's queries, side by side
     if (tid < nq) {
         qu[tid] = standardise(m.xform[F - 2], q.in_len[q0 + tid], m.mu[F - 2], m.sd[F - 2]);
     } else if (tid >= 32 && tid < 32 + nq) {
@@ -1821,8 +1820,8 @@ __device__ __forceinline__ void pair_cols_fused(const Model &m, const Queries &q
     float *w2c = sm + L.w2;    // [cols][ldk]: W2 rows n0 .. n0 + cols - 1
     float *as = sm + L.as;     // [PAIR_G][lda]: each pair's deployment prefix
     float *w1s = sm + L.w1;    // [2][ldk]: W1's two query columns
-    // the query slots' raw lengths first: their double-precision chains below
-    // are this block's longest wait
+    // the query slots' raw lengths first: what follows from them below is this
+    // block's longest wait
     float iv = 0.f, ov = 0.f;
     if (tid < nq) iv = q.in_len[q0 + tid];
     else if (tid >= 32 && tid < 32 + nq) ov = q.out_len[q0 + tid - 32];
@@ -1873,7 +1872,7 @@ __device__ __forceinline__ void pair_cols_fused(const Model &m, const Queries &q
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     }
-    // the query slots of the group's queries (fp64 chains side by side)
+    // the query slots of the group's queries, side by side
     if (tid < nq) {
         qu[tid] = standardise(m.xform[F - 2], iv, m.mu[F - 2], m.sd[F - 2]);
     } else if (tid >= 32 && tid < 32 + nq) {
