@@ -910,9 +910,19 @@ k_route_rows(Model m, Queries q, int32_t *status) {
                     }
             }
             __syncwarp();
-            // the groups that the last block does not have
-            if (blk == nblk - 1 && lane == 0)
-                for (int g = last_groups; g < G; ++g) umma::mbar_arrive(&done[slot]);
+            // the groups that the last block does not have arrive from here, once
+            // the slot is this block's: the block NB before it, another deciding
+            // warp's, may still be waiting for its own groups
+            if (blk == nblk - 1 && last_groups < G) {
+                if (blk >= NB) {
+                    ok = umma::mbar_wait(&freed[slot], ((blk / NB) & 1) ^ 1, abort_f, status);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
+                }
+                if (lane == 0)
+                    for (int g = last_groups; g < G; ++g) umma::mbar_arrive(&done[slot]);
+                __syncwarp();
+            }
             ok = umma::mbar_wait(&done[slot], (blk / NB) & 1, abort_f, status);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
@@ -2254,8 +2264,15 @@ static cudaError_t launch_rows(const Model &m, const Queries &q, int nsm, int32_
 // 24,000 22.9 / 31.2, 48,000 39.4 / 36.9, 1.2 M 760 / 396; H = 32: 48,000
 // 31.4 / 33.1, 96,000 57.9 / 35.2, 1.2 M 610 / 236; H = 256: 18,000 71.2 /
 // 82.6, 30,000 134 / 103, 240,000 850 / 756.
+// With few deployments a query's quality chains weigh more, and at 65 to 128
+// columns (two deciding warps) they bound k_route_rows: up to 4 deployments it
+// gains nothing there (D = 4, E = 1024: 40,000 pairs 80 / 92, 320,000 434 /
+// 442), up to 7 from about three rounds on (D = 6, E = 1024: 60,000 97 / 102,
+// 120,000 175 / 161).
 static bool rows_kernel(const Model &m, int Q, int nsm) {
-    return (long)Q * m.D > 64L * (m.H2 <= 128 ? 3 : 2) * nsm;
+    const long pairs = (long)Q * m.D, round = 64L * (m.H2 <= 128 ? 3 : 2) * nsm;
+    if (m.H2 > 64 && m.H2 <= 128 && m.D < 8) return m.D > 4 && pairs > 3 * round;
+    return pairs > round;
 }
 
 cudaError_t launch_route_simt(const Model &m, const Queries &q, int nsm, int32_t *status,

@@ -39,7 +39,12 @@ CASES = [
     (2433, 4, 3, 64, 33, 8, "f32", 2),
     (4871, 3, 2, 50, 64, 96, "f32", 3),
     (2440, 4, 3, 128, 128, 72, "f32", 2),
+    (80003, 1, 1, 64, 64, 64, "f32", 2),      # few groups a query block: several blocks a pass
+    (80003, 1, 1, 32, 20, 8, "f32", 3),
+    (40010, 2, 1, 48, 200, 64, "f32", 2),
+    (17600, 5, 1, 96, 128, 104, "f32", 2),
     (1950, 5, 3, 129, 96, 104, "f32", 3),
+    (9003, 9, 1, 64, 100, 512, "f32", 2),
     (700, 9, 5, 160, 65, 64, "f32", 2),
     (1470, 20, 1, 40, 128, 32, "f32", 2),
     (900, 33, 1, 100, 70, 48, "f32", 3),
