@@ -2269,6 +2269,8 @@ static cudaError_t launch_rows(const Model &m, const Queries &q, int nsm, int32_
 // gains nothing there (D = 4, E = 1024: 40,000 pairs 80 / 92, 320,000 434 /
 // 442), up to 7 from about three rounds on (D = 6, E = 1024: 60,000 97 / 102,
 // 120,000 175 / 161).
+// At up to 64 columns the line stays: D = 4, E = 1024 loses only around 80,000
+// pairs (H = 32 85 / 91, H = 64 93 / 98) and gains at 40,000 and from 160,000 on.
 static bool rows_kernel(const Model &m, int Q, int nsm) {
     const long pairs = (long)Q * m.D, round = 64L * (m.H2 <= 128 ? 3 : 2) * nsm;
     if (m.H2 > 64 && m.H2 <= 128 && m.D < 8) return m.D > 4 && pairs > 3 * round;
