@@ -910,15 +910,16 @@ k_route_rows(Model m, Queries q, int32_t *status) {
                     }
             }
             __syncwarp();
-            // the groups that the last block does not have arrive from here, once
-            // the slot is this block's: the block NB before it, another deciding
-            // warp's, may still be waiting for its own groups
+            // The slot is this block's once the block NB before it is decided; that
+            // one may be another deciding warp's and still wait for its groups, and
+            // `done` would then be a phase behind, whose parity reads as complete.
+            if (blk >= NB) {
+                ok = umma::mbar_wait(&freed[slot], ((blk / NB) & 1) ^ 1, abort_f, status);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+            }
+            // the groups that the last block does not have arrive from here
             if (blk == nblk - 1 && last_groups < G) {
-                if (blk >= NB) {
-                    ok = umma::mbar_wait(&freed[slot], ((blk / NB) & 1) ^ 1, abort_f, status);
-                    ok = __all_sync(0xffffffffu, ok);
-                    if (!ok) break;
-                }
                 if (lane == 0)
                     for (int g = last_groups; g < G; ++g) umma::mbar_arrive(&done[slot]);
                 __syncwarp();

@@ -42,6 +42,13 @@ CASES = [
     (80003, 1, 1, 64, 64, 64, "f32", 2),      # few groups a query block: several blocks a pass
     (80003, 1, 1, 32, 20, 8, "f32", 3),
     (40010, 2, 1, 48, 200, 64, "f32", 2),
+    # short quality chains: a deciding warp is ready before the block that had
+    # its cost slot is scored
+    (94987, 1, 1, 128, 16, 48, "f32", 3),
+    (70001, 2, 1, 160, 64, 8, "f32", 2),
+    (60007, 1, 3, 256, 33, 8, "f32", 3),
+    (50021, 4, 1, 128, 64, 8, "f32", 2),
+    (40009, 5, 1, 200, 40, 16, "bf16", 2),
     (17600, 5, 1, 96, 128, 104, "f32", 2),
     (1950, 5, 3, 129, 96, 104, "f32", 3),
     (9003, 9, 1, 64, 100, 512, "f32", 2),
