@@ -551,8 +551,8 @@ k_route_simt(Model m, Queries q, HostFlag flag) {
 // the warp tile; NQ warps hold one query per lane and, a block of queries
 // ahead of the tile, run its quality chains, then wait for the block's costs
 // and decide.  The costs pass through a ring of NB blocks in shared memory
-// (mbarriers: done, a group's arrival; freed, the decision's), so the two
-// sides meet only when one is a whole ring ahead.
+// (done, an mbarrier: the groups' arrivals; freed, a count: the decisions), so
+// the two sides meet only when one is a whole ring ahead.
 // Bound: the FMA pipe; measured 42.5 TFLOP/s at 100,000 queries, D = 12,
 // H = 128 (53 % of 80.5; k_route_simt 31), where a k step's 64 packed FMAs
 // come with about 50 other instructions (the pairs of a W2 value with itself,
@@ -613,7 +613,7 @@ __host__ __device__ inline RowsLayout rows_layout(int D, int M, int NH, int H1, 
     L.qst = take((size_t)S::NQ * S::QST * L.qst_bytes);
     L.qual = take((size_t)S::NQ * L.qbk * (M | 1) * 4);
     L.dms = take((size_t)D * 4);
-    L.bars = take((S::NS + 2 * S::NB) * 8 + (S::NS + 2) * 4);
+    L.bars = take((S::NS + S::NB) * 8 + (S::NB + S::NS + 2) * 4);
     // W2 stages: as many as fit, all of it if possible (and slack: the widest
     // lane reads past a row that ends before W)
     const size_t stage = (size_t)TILE_KC * H2p * 4;
@@ -675,6 +675,34 @@ __device__ __forceinline__ void qual_chunk(const char *row, const float *mb, int
     }
 }
 
+// A cost slot's count of decisions: its deciding warps say that the n-th use is
+// over; the others wait for it.  A count and not an mbarrier's phase: with few
+// deployments a pass of the scoring warps spans more blocks than the ring has,
+// a warp then comes to a slot that it has not seen for two uses, and the
+// parity of the phase before last reads like that of the last one.
+__device__ __forceinline__ void slot_free(uint32_t *freed, uint32_t n) {
+    asm volatile("st.release.cta.shared.u32 [%0], %1;" ::"r"(umma::smem_u32(freed)), "r"(n) : "memory");
+}
+
+__device__ __forceinline__ bool slot_wait(const uint32_t *freed, uint32_t n, volatile int *abort_f,
+                                          int32_t *status) {
+    const uint32_t a = umma::smem_u32(freed);
+    const long long t0 = clock64();
+    while (true) {
+        uint32_t v;
+        asm volatile("ld.acquire.cta.shared.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+        if (v >= n) return true;
+        if (*abort_f) return false;
+        if (clock64() - t0 > umma::WAIT_CYCLES) {
+            *abort_f = 1;
+            *(volatile int32_t *)status = ST_TIMEOUT;
+            __threadfence_system();
+            return false;
+        }
+        __nanosleep(64);
+    }
+}
+
 template <int W>
 __global__ void __launch_bounds__(RouteShape<W>::THREADS, 1)
 k_route_rows(Model m, Queries q, int32_t *status) {
@@ -696,9 +724,8 @@ k_route_rows(Model m, Queries q, int32_t *status) {
     const int ngroups = nblk ? (nblk - 1) * G + last_groups : 0;
     const int passes = (ngroups + NW - 1) / NW;
 
-    uint64_t *full = reinterpret_cast<uint64_t *>(sm + L.bars), *done = full + S::NS,
-             *freed = done + NB;
-    uint32_t *used = reinterpret_cast<uint32_t *>(freed + NB);
+    uint64_t *full = reinterpret_cast<uint64_t *>(sm + L.bars), *done = full + S::NS;
+    uint32_t *freed = reinterpret_cast<uint32_t *>(done + NB), *used = freed + NB;
     volatile int *abort_f = reinterpret_cast<volatile int *>(used + S::NS);
     W2Feed f;
     f.w2t = m.W2T;
@@ -721,7 +748,7 @@ k_route_rows(Model m, Queries q, int32_t *status) {
         }
         for (int b = 0; b < NB; ++b) {
             umma::mbar_init(&done[b], G);
-            umma::mbar_init(&freed[b], 1);
+            freed[b] = 0;
         }
         *abort_f = 0;
         umma::fence_mbar_init();
@@ -796,7 +823,7 @@ k_route_rows(Model m, Queries q, int32_t *status) {
             // the block's slot is free once the decisions NB blocks back are out
             const int blk = g / G, slot = blk % NB;
             if (blk >= NB) {
-                const bool ok = umma::mbar_wait(&freed[slot], ((blk / NB) & 1) ^ 1, abort_f, status);
+                const bool ok = slot_wait(&freed[slot], (uint32_t)(blk / NB), abort_f, status);
                 if (!__all_sync(0xffffffffu, ok)) break;
             }
             if (lane < RG && cq >= 0) {
@@ -914,7 +941,7 @@ k_route_rows(Model m, Queries q, int32_t *status) {
             // one may be another deciding warp's and still wait for its groups, and
             // `done` would then be a phase behind, whose parity reads as complete.
             if (blk >= NB) {
-                ok = umma::mbar_wait(&freed[slot], ((blk / NB) & 1) ^ 1, abort_f, status);
+                ok = slot_wait(&freed[slot], (uint32_t)(blk / NB), abort_f, status);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
             }
@@ -950,7 +977,7 @@ k_route_rows(Model m, Queries q, int32_t *status) {
                 if (better(o, best)) best = o;
             }
             __syncwarp();
-            if (lane == 0) umma::mbar_arrive(&freed[slot]);
+            if (lane == 0) slot_free(&freed[slot], (uint32_t)(blk / NB) + 1u);
             if (valid && half == 0) {
                 const bool sel = best.cls > 0;
                 q.chosen[qq] = sel ? best.d : -1;

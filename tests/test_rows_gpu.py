@@ -42,6 +42,11 @@ CASES = [
     (80003, 1, 1, 64, 64, 64, "f32", 2),      # few groups a query block: several blocks a pass
     (80003, 1, 1, 32, 20, 8, "f32", 3),
     (40010, 2, 1, 48, 200, 64, "f32", 2),
+    # a pass of the scoring warps spans more query blocks than the cost ring,
+    # and long quality chains keep the decisions behind
+    (60001, 1, 1, 40, 136, 1024, "f32", 2),
+    (60001, 1, 1, 8, 130, 2048, "bf16", 3),
+    (30003, 2, 1, 20, 132, 2048, "f32", 2),
     # short quality chains: a deciding warp is ready before the block that had
     # its cost slot is scored
     (94987, 1, 1, 128, 16, 48, "f32", 3),
