@@ -129,12 +129,18 @@ struct hwr_ctx {
     uint32_t simt_blocks = 0;
     int32_t flag_seq = 0;
     bool want_flag = false, flagged = false;    // this call wants one; its kernel sets one
-    // outputs of the last tensor-core route (its predictor may still run
-    // while the next route's kernels start)
+    // outputs of the tensor-core routes that may still be running: every queued
+    // route's kernels start before those of the routes before it have finished,
+    // any number of routes deep (as many as find SMs), so all of them are kept
+    // until a kernel that waits for them, or the host, has seen them complete
     struct Range {
-        const void *p = nullptr;
-        size_t n = 0;
-    } prev_out[5];                   // chosen, latency, utility, per-pair costs, quality
+        const void *p;
+        size_t n;
+    };
+    static constexpr int LIVE_MAX = 96, ROUTE_OUTPUTS = 5;   // a route: chosen, latency, utility,
+                                                             // per-pair costs, quality
+    Range live[LIVE_MAX];
+    int n_live = 0;
     // a snapshot kernel may still read the staging: set at its launch, cleared
     // once the host has seen later work on the stream complete
     bool snap_busy = false;
@@ -699,6 +705,7 @@ extern "C" hwr_status hwr_update_snapshot(hwr_ctx *c, const hwr_snapshot *s) {
     ls.done();
     CK(c, cudaEventRecord(c->snap_ev, c->stream), "record");
     c->snap_busy = true;
+    c->n_live = 0;      // (a plain launch: it starts when every kernel before has finished)
     c->have_snapshot = true;
     return HWR_OK;
 }
@@ -722,6 +729,25 @@ extern "C" hwr_status hwr_get_snapshot(hwr_ctx *c, int32_t *running_out) {
 static bool overlaps(const void *a, size_t na, const void *b, size_t nb) {
     const uintptr_t x = (uintptr_t)a, y = (uintptr_t)b;
     return a && b && na && nb && x < y + nb && y < x + na;
+}
+
+// Whether bytes [p, p + n) touch an output of a route that may still be running.
+static bool overlaps_live(const hwr_ctx *c, const void *p, size_t n) {
+    for (int i = 0; i < c->n_live; ++i)
+        if (overlaps(p, n, c->live[i].p, c->live[i].n)) return true;
+    return false;
+}
+
+// Room for ROUTE_OUTPUTS more must be there.  (A caller's buffers come round
+// again: ranges that an entry covers are not added.)
+static void add_live(hwr_ctx *c, const void *p, size_t n) {
+    if (!p || !n) return;
+    const uintptr_t a = (uintptr_t)p;
+    for (int i = 0; i < c->n_live; ++i) {
+        const uintptr_t b = (uintptr_t)c->live[i].p;
+        if (a >= b && a + n <= b + c->live[i].n) return;
+    }
+    c->live[c->n_live++] = {p, n};
 }
 
 static hwr_status run_kernels(hwr_ctx *c, const Queries &q, uint32_t flags, bool tensor) {
@@ -847,29 +873,31 @@ static hwr_status run_kernels(hwr_ctx *c, const Queries &q, uint32_t flags, bool
         }
         // The predictor may start as soon as the quality kernel has: before
         // its dependency wait it reads only weights, the snapshot's prefixes
-        // and this call's inputs -- unless those inputs are outputs of the
-        // previous tensor-core route, whose predictor may still be running.
+        // and this call's inputs -- unless those inputs are outputs of earlier
+        // tensor-core routes, whose predictors may still be running.  (The
+        // quality kernel reads the embeddings at once: over such outputs, or with
+        // no room to note this call's, it waits for the kernels before
+        // altogether.)  A predictor that does not start early starts when every
+        // kernel before has finished, and so do all that follow it.
         const size_t qb4 = (size_t)q.Q * 4;
-        // (The quality kernel reads the embeddings at once: over earlier outputs
-        // it waits for the kernels before altogether.)
-        bool early = true, dependent = true;
-        for (const auto &o : c->prev_out) {
-            if (overlaps(q.emb, (size_t)q.Q * c->E * 2, o.p, o.n)) dependent = false;
-            if (!dependent || overlaps(q.in_len, qb4, o.p, o.n) || overlaps(q.out_len, qb4, o.p, o.n) ||
-                (q.slo_q && overlaps(q.slo_q, qb4, o.p, o.n)))
-                early = false;
-        }
+        const bool dependent = c->n_live + hwr_ctx::ROUTE_OUTPUTS <= hwr_ctx::LIVE_MAX &&
+                               !overlaps_live(c, q.emb, (size_t)q.Q * c->E * 2);
+        const bool early = dependent && !overlaps_live(c, q.in_len, qb4) &&
+                           !overlaps_live(c, q.out_len, qb4) && !overlaps_live(c, q.slo_q, qb4);
+        if (!early) c->n_live = 0;
         const int free_sms = tc_mlp_free_sms(q.Q, sp);
         LaunchScope a(c, HWR_K_QUAL_TC, prof);
         CK(c, launch_qual_tc(t, q, qb, c->status_d, c->stream, dependent, early, free_sms, c->done_d,
                              c->pred_ctas - c->pred_ctas_last, q.qual_out),
            "quality kernel");
         a.done();
-        c->prev_out[0] = {q.chosen, qb4};
-        c->prev_out[1] = {q.lat, qb4};
-        c->prev_out[2] = {q.util, qb4};
-        c->prev_out[3] = {q.pair_C, q.pair_C ? qb4 * c->D : 0};
-        c->prev_out[4] = {q.qual_out, q.qual_out ? qb4 * c->M : 0};
+        if (!q.no_select) {
+            add_live(c, q.chosen, qb4);
+            add_live(c, q.lat, qb4);
+            add_live(c, q.util, qb4);
+        }
+        add_live(c, q.pair_C, qb4 * c->D);
+        add_live(c, q.qual_out, qb4 * c->M);
         LaunchScope b(c, HWR_K_MLP_TC, prof);
         int ctas = 0;
         HostFlag flag;
@@ -1245,6 +1273,7 @@ static hwr_status route_impl(hwr_ctx *c, int32_t Q, const float *in_len, const f
     // this call's work is complete, and with it every earlier kernel
     c->async_pending = false;
     c->snap_busy = false;
+    c->n_live = 0;
     CK(c, cudaGetLastError(), "kernel");
     return check_status_word(c);
 }
@@ -1308,6 +1337,7 @@ extern "C" hwr_status hwr_synchronize(hwr_ctx *c) {
     CK(c, cudaStreamSynchronize(c->stream), "synchronize");
     c->async_pending = false;
     c->snap_busy = false;
+    c->n_live = 0;
     return check_status_word(c);
 }
 
@@ -1393,13 +1423,13 @@ hwr_status hwr_internal_route_tensor_scratch(hwr_ctx *c, int32_t Q, const float 
     CK(c, launch_mlp_tc(t, q, qual, sp, part, count, c->status_d, c->stream, nullptr, &ctas),
        "predictor kernel");
     // this predictor may still run when the next tensor-core route starts
-    // early: that route checks its inputs against these outputs
+    // early: that route checks its inputs against these outputs (the plain
+    // launch above waited for every kernel before)
     const size_t qb4 = (size_t)Q * 4;
-    c->prev_out[0] = {chosen, qb4};
-    c->prev_out[1] = {pred_latency, qb4};
-    c->prev_out[2] = {utility, qb4};
-    c->prev_out[3] = {};
-    c->prev_out[4] = {};
+    c->n_live = 0;
+    add_live(c, chosen, qb4);
+    add_live(c, pred_latency, qb4);
+    add_live(c, utility, qb4);
     c->stats.kernel_launches++;
     c->stats.launches[HWR_K_MLP_TC]++;
     c->stats.queries_routed += Q;
