@@ -77,7 +77,7 @@ struct hwr_ctx {
     int test_stall = 0;          // HWR_TEST_STALL: tensor-path producers never signal
     int tc_min_pairs = TC_MIN_PAIRS, pairs_max = -1;   // -1: by the context's paths
     int device = -1;             // the CUDA device current at hwr_create
-    long poll_us = 1000000;      // small-batch output poll limit (HWR_TEST_POLL_US)
+    long poll_us = 1000000;      // limit of the host's polls (HWR_TEST_POLL_US)
     bool async_pending = false;  // an HWR_ASYNC call may still have work queued
     // the GPU reads and writes pageable host memory coherently (address
     // translation services over the CPU-GPU link, as on Grace + GB300):
@@ -953,6 +953,13 @@ static bool wait_chosen(const int32_t *ch, int Q, long limit_us) {
     return true;
 }
 
+// The host word of a waited device call is polled for this long at most, then
+// the stream is synchronised: behind long work that the caller has queued on
+// its own stream the host holds a core no longer than that (asking the stream
+// first would cost 0.7 us, what the word saves), and a longer call loses
+// under 1 % by the synchronisation.
+constexpr long FLAG_POLL_US = 150;
+
 // The host word of a waited device call; false after limit_us.
 static bool wait_flag(const int32_t *word, int32_t value, long limit_us) {
     const auto t0 = std::chrono::steady_clock::now();
@@ -1133,9 +1140,15 @@ static hwr_status route_impl(hwr_ctx *c, int32_t Q, const float *in_len, const f
     // A waited route on device pointers: its kernel's last block sets a host
     // word, and the host waits for that instead of synchronising the stream
     // (256 fp32 queries at D = 4: 20.5 -> 19.2 us; 4,096 bf16 ones at D = 12:
-    // 28.3 -> 27.6)
+    // 28.3 -> 27.6), unless an HWR_ASYNC call's work is still running, as above
     c->want_flag = dev && !seq && !ml && !so && !(flags & (HWR_ASYNC | HWR_PROFILE)) && c->poll_us > 0;
     c->flagged = false;
+    if (c->want_flag && c->async_pending) {
+        const cudaError_t e = cudaStreamQuery(c->stream);
+        if (e != cudaSuccess && e != cudaErrorNotReady) return cuda_fail(c, e, "query stream");
+        c->async_pending = e == cudaErrorNotReady;
+        c->want_flag = !c->async_pending;
+    }
     if (c->want_flag) {
         c->flag_seq = c->flag_seq == INT32_MAX ? 1 : c->flag_seq + 1;
         __atomic_store_n(c->flag_h, 0, __ATOMIC_RELAXED);
@@ -1268,7 +1281,8 @@ static hwr_status route_impl(hwr_ctx *c, int32_t Q, const float *in_len, const f
         c->async_pending = true;
         return HWR_OK;
     }
-    if (!synced && !(c->flagged && wait_flag(c->flag_h, c->flag_seq, c->poll_us)))
+    if (!synced && !(c->flagged && wait_flag(c->flag_h, c->flag_seq,
+                                             c->poll_us < FLAG_POLL_US ? c->poll_us : FLAG_POLL_US)))
         CK(c, cudaStreamSynchronize(c->stream), "synchronize");
     // this call's work is complete, and with it every earlier kernel
     c->async_pending = false;
