@@ -2320,18 +2320,19 @@ cudaError_t launch_route_simt(const Model &m, const Queries &q, int nsm, int32_t
     const RouteLayout L = route_layout(m.D, m.M, m.H2);
     const int blocks = (q.Q + L.QB - 1) / L.QB;
     const size_t smem = L.total * sizeof(float);
-    if (flag.word) {
-        *blocks_done += (uint32_t)blocks;
-        flag.target = *blocks_done;
-        *flagged = true;
-    }
+    if (flag.word) flag.target = *blocks_done + (uint32_t)blocks;
     switch (cpt_for(m.H2)) {
         case 1: k_route_simt<1><<<blocks, ROUTE_THREADS, smem, s>>>(m, q, flag); break;
         case 2: k_route_simt<2><<<blocks, ROUTE_THREADS, smem, s>>>(m, q, flag); break;
         case 4: k_route_simt<4><<<blocks, ROUTE_THREADS, smem, s>>>(m, q, flag); break;
         default: k_route_simt<8><<<blocks, ROUTE_THREADS, smem, s>>>(m, q, flag); break;
     }
-    return cudaGetLastError();
+    const cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess && flag.word) {      // (a launch that failed counts no blocks)
+        *blocks_done = flag.target;
+        *flagged = true;
+    }
+    return e;
 }
 
 size_t route_pairs_smem(const Model &m) {
