@@ -771,10 +771,16 @@ static hwr_status run_kernels(hwr_ctx *c, const Queries &q, uint32_t flags, bool
             TRY(grow(c, &c->qual, &c->qual_cap, 2 * (size_t)Qs * c->Mpad));
         }
         TRY(grow(c, &c->ctab, &c->ctab_cap, seq_table_floats(c->D, Qs)));
-        // (SIMT table: whole chunks whose prefixes are prepared at once)
-        const int run = tcs ? Qs : (SEQ_RUN / Qs > 1 ? SEQ_RUN / Qs : 1) * Qs;
-        TRY(grow(c, &c->qseq, &c->qseq_cap,
-                 seq_aux_floats(c->D, c->M, c->H1, run < q.Q ? run : q.Q)));
+        // (SIMT table: whole chunks whose prefixes are prepared at once, D (run + 1) H1
+        // floats, 84 MB at the largest shape; without the memory for them, one chunk's)
+        int run = tcs ? Qs : (SEQ_RUN / Qs > 1 ? SEQ_RUN / Qs : 1) * Qs;
+        if (run > q.Q) run = q.Q;
+        hwr_status room = grow(c, &c->qseq, &c->qseq_cap, seq_aux_floats(c->D, c->M, c->H1, run));
+        if (room == HWR_ERR_OOM && run > Qs) {
+            run = Qs;
+            room = grow(c, &c->qseq, &c->qseq_cap, seq_aux_floats(c->D, c->M, c->H1, run));
+        }
+        TRY(room);
         int run_lo = 0, run_n = 0;
         const size_t es = c->dtype == HWR_BF16 ? 2 : 4;
         for (int lo = 0; lo < q.Q; lo += Qs) {
