@@ -14,7 +14,9 @@
 // (whose own error is 2^-51).  Otherwise, about once in 2^15 softplus values
 // (1,451 of 2^26), and for arguments outside the ranges below, the
 // double-precision evaluation runs.  The result is the same float for every
-// argument (checked for all 2^32 of them by the tests).
+// argument: the tests check softplus and sigmoid for all 2^32 of them,
+// standardisation for all 2^32 under several constants and for random
+// constants on a sample.
 //
 // Series: exp by its Taylor polynomial after a reduction by multiples of ln 2
 // (held in three parts, so that the reduction is exact); log(m) =
@@ -167,11 +169,27 @@ static __device__ __noinline__ float sigmoid_dp(float s) {
 // arguments in [-12, 12]: exp and softplus 2^-41.1, log 2^-44.1.
 constexpr float FF_ERR = 0x1p-40f, FF_LOG_ERR = 0x1p-42f;
 
+// (t - mu) / sd as q + l, and a bound on the error of rounding q + l +- err (t is
+// off by terr at most).  With u = 2^-24 and r the remainder d - q sd: q is off
+// by u from its product and 2 u from the reciprocal, so |r / sd| <= 3 u |q|; l
+// takes one rounding of r and of d.l + t.l each, of their sum and of the
+// product, and the reciprocal's 2 u, in all at most 5 u |l| + 6 u^2 |q|; adding
+// err to l rounds once more, u |l|.  6 u |l| + 6 u^2 |q| is under 2^-21 |l| +
+// 2^-43 |q|.  (2^-42 |q| alone does not always bracket the value where |l| comes
+// near 2^-20 |q|, which only counts past 2^24 reach.)
+__device__ __forceinline__ ff ff_standard(ff t, float terr, float mu, float sd, float *err) {
+    const ff d = two_sum(t.h, -mu);
+    const float rc = rcp_approx(sd), q = d.h * rc;
+    const ff x{q, (__fmaf_rn(-q, sd, d.h) + (d.l + t.l)) * rc};
+    *err = terr * fabsf(rc) + __fmaf_rn(0x1p-21f, fabsf(x.l), 0x1p-43f * fabsf(q));
+    return x;
+}
+
 // (t(raw) - mu) / sd with the slot transform t: 0 identity, 1 log1p, 2 log.
 // raw = rh + rl exactly (rl is non-zero for integers past 2^24 only).
 __device__ __forceinline__ float standardise(uint8_t code, ff raw, float mu, float sd) {
     ff t = raw;
-    float err = 0.f;
+    float terr = 0.f;
     bool ok = true;
     if (code) {
         ff w = raw;
@@ -182,19 +200,19 @@ __device__ __forceinline__ float standardise(uint8_t code, ff raw, float mu, flo
         }
         ok = ok && w.h >= 0x1p-40f && w.h <= 0x1p40f;
         t = ff_log(w);
-        err = FF_LOG_ERR * fabsf(t.h) + 0x1p-48f;
+        terr = FF_LOG_ERR * fabsf(t.h) + 0x1p-48f;
     }
-    const ff d = two_sum(t.h, -mu);
-    const float rc = rcp_approx(sd), q = d.h * rc;
-    const ff x{q, (__fmaf_rn(-q, sd, d.h) + (d.l + t.l)) * rc};
+    float err;
+    const ff x = ff_standard(t, terr, mu, sd, &err);
+    const float q = x.h;
     ok = ok && fabsf(sd) >= 0x1p-40f && fabsf(sd) <= 0x1p40f;
     // an exact zero: the quotient is a zero of the right sign
-    if (ok && d.h == 0.f && x.l == 0.f && err == 0.f) return q;
+    if (ok && t.h == mu && x.l == 0.f && terr == 0.f) return q;
     // the quotient far from the ends of the float range, its low part small
     // (it is computed in single)
     ok = ok && fabsf(q) >= 0x1p-40f && fabsf(q) <= 0x1p60f && fabsf(x.l) <= 0x1p-20f * fabsf(q);
     float r;
-    if (ok && ff_round(x, err * fabsf(rc) + 0x1p-42f * fabsf(q), &r)) return r;
+    if (ok && ff_round(x, err, &r)) return r;
     return standardise_dp(code, raw.h, raw.l, mu, sd);
 }
 

@@ -1,8 +1,9 @@
 """The two-float transcendental functions (canon_math.cuh) against their
 double-precision definitions, bit for bit: softplus and sigmoid for every
 float, standardisation for every float under each transform with the
-constants of a predictor, and for counts and other constants on a sample
-around the values where the evaluation changes its way."""
+constants of a predictor, and for counts and other constants (random ones among
+them) on a sample around the values where the evaluation changes its way; and
+the bound on the quotient's error where it is tightest."""
 import importlib
 import os
 import subprocess
@@ -59,6 +60,58 @@ __global__ void counts(int code, float mu, float sd, unsigned long long *bad) {
     if (b) atomicAdd(bad, b);
 }
 
+__device__ unsigned long long next(unsigned long long &s) {
+    s ^= s << 13;
+    s ^= s >> 7;
+    s ^= s << 17;
+    return s;
+}
+
+// random constants of any size and sign, arguments near and far from the mean,
+// counts among them
+__global__ void random_constants(int code, unsigned long long *bad) {
+    unsigned long long s = 88172645463325252ull + 2 * (blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x), b = 0;
+    for (int k = 0; k < 20; ++k) next(s);
+    for (int k = 0; k < 512; ++k) {
+        const unsigned long long u = next(s), v = next(s), w = next(s);
+        const float sd = __int_as_float((int)((unsigned)(v & 0x807fffffu) | (unsigned)(97 + (v >> 32) % 60) << 23));
+        const float m = __int_as_float((int)((unsigned)(w & 0x007fffffu) | (unsigned)(87 + (w >> 32) % 60) << 23));
+        const int i = (int)((u >> 8) & 0x7fffffffu) >> (u & 31);
+        const ff c = u & 128 ? ff_count(i) : ff{m * (1.f + (float)((int)(u >> 40) - (1 << 23)) * 0x1p-30f), 0.f};
+        const double raw = (double)c.h + (double)c.l;
+        double t = raw;
+        if (code == 1) t = log1p(raw);
+        else if (code == 2) t = log(raw);
+        const float mu = u & 64 ? (float)t * (w & (1u << 30) ? 1.f : 1.0001f) : m * (w & (1u << 30) ? 1.f : -1.f);
+        b += !same(standardise((uint8_t)code, c, mu, sd), (float)((t - (double)mu) / (double)sd));
+    }
+    if (b) atomicAdd(bad, b);
+}
+
+// what the rounding test needs of the quotient: the two sums it compares lie on
+// either side of the value, here for counts past 2^24 whose distance from the
+// mean lets the low part reach its limit
+__global__ void brackets(unsigned long long *bad) {
+    unsigned long long s = 88172645463325252ull + 2 * (blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x), b = 0;
+    for (int k = 0; k < 20; ++k) next(s);
+    for (int k = 0; k < 4096; ++k) {
+        const unsigned long long u = next(s), v = next(s);
+        const int i = (1 << 24) + (int)(v % (u & 1 ? 1u << 28 : 0x7effffffu));
+        const ff c = ff_count(i);
+        if (c.l == 0.f) continue;
+        const float d = fabsf(c.l) * 0x1p20f * (1.f + (float)(u >> 54) * 0x1p-12f);
+        const float mu = u & 2 ? c.h - d : c.h + d;
+        const float sd = __int_as_float(0x3f800000 | (int)((u >> 8) & 0x7fffff));
+        float err;
+        const ff x = ff_standard(c, 0.f, mu, sd, &err);
+        if (fabsf(x.l) > 0x1p-20f * fabsf(x.h)) continue;
+        const double want = ((double)i - (double)mu) / (double)sd;
+        const float up = x.l + err, dn = x.l - err;
+        b += !((double)x.h + (double)up >= want && (double)x.h + (double)dn <= want);
+    }
+    if (b) atomicAdd(bad, b);
+}
+
 int main(int argc, char **argv) {
     const int op = atoi(argv[1]);
     const float mu = argc > 2 ? (float)atof(argv[2]) : 0.f, sd = argc > 3 ? (float)atof(argv[3]) : 1.f;
@@ -66,7 +119,9 @@ int main(int argc, char **argv) {
     cudaMalloc(&d, 8);
     cudaMemcpy(d, &h, 8, cudaMemcpyHostToDevice);
     if (op < 10) all<<<152 * 8, 256>>>(op, mu, sd, d);
-    else counts<<<152 * 8, 256>>>(op - 10, mu, sd, d);
+    else if (op < 20) counts<<<152 * 8, 256>>>(op - 10, mu, sd, d);
+    else if (op < 30) random_constants<<<152 * 8, 256>>>(op - 20, d);
+    else brackets<<<152 * 8, 256>>>(d);
     cudaMemcpy(&h, d, 8, cudaMemcpyDeviceToHost);
     printf("%s %llu\n", cudaGetErrorString(cudaGetLastError()), h);
     return 0;
@@ -107,3 +162,12 @@ CONSTANTS = [(5.5099, 0.99718), (-2.0006, 0.49971), (2.0738, 0.39), (0.4, 0.2), 
 def test_standardise_for_every_float_and_count(prog, code, mu, sd):
     _run(prog, 2 + code, mu, sd)
     _run(prog, 10 + code, mu, sd)
+
+
+@pytest.mark.parametrize("code", [0, 1, 2])
+def test_standardise_for_random_constants(prog, code):
+    _run(prog, 20 + code)
+
+
+def test_the_quotient_stays_within_its_bound(prog):
+    _run(prog, 30)
