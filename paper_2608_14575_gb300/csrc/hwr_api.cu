@@ -76,6 +76,7 @@ struct hwr_ctx {
     bool have_snapshot = false;
     int test_stall = 0;          // HWR_TEST_STALL: tensor-path producers never signal
     int tc_min_pairs = TC_MIN_PAIRS, pairs_max = -1;   // -1: by the context's paths
+    int batch_kernel = -1;       // HWR_TEST_BATCH_KERNEL: the fp32 batch kernel (launch_route_simt)
     int device = -1;             // the CUDA device current at hwr_create
     long poll_us = 1000000;      // limit of the host's polls (HWR_TEST_POLL_US)
     bool async_pending = false;  // an HWR_ASYNC call may still have work queued
@@ -640,6 +641,7 @@ extern "C" hwr_status hwr_create(const hwr_deployment_table *table, const hwr_pr
         c->ats = pageable == 1 && !(h && atoi(h) != 0);
     }
     if (const char *h = getenv("HWR_TEST_STALL")) c->test_stall = atoi(h) != 0;
+    if (const char *h = getenv("HWR_TEST_BATCH_KERNEL")) c->batch_kernel = atoi(h) == 1 ? 1 : 0;
     if (const char *h = getenv("HWR_TC_MIN_PAIRS")) c->tc_min_pairs = atoi(h) > 1 ? atoi(h) : 1;
     if (const char *h = getenv("HWR_PAIRS_MAX_PAIRS"))
         c->pairs_max = atoi(h) < 0 ? 0 : (atoi(h) > PAIRS_MAX_PAIRS ? PAIRS_MAX_PAIRS : atoi(h));
@@ -933,7 +935,7 @@ static hwr_status run_kernels(hwr_ctx *c, const Queries &q, uint32_t flags, bool
             flag.count = c->simt_done_d;
             flag.value = c->flag_seq;
         }
-        CK(c, launch_route_simt(m, q, c->nsm, c->status_d, flag, &c->simt_blocks, &c->flagged,
+        CK(c, launch_route_simt(m, q, c->nsm, c->batch_kernel, c->status_d, flag, &c->simt_blocks, &c->flagged,
                                 c->stream), "route kernel");
     }
     a.done();

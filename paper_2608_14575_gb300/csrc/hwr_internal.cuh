@@ -137,11 +137,12 @@ __device__ __forceinline__ void flag_block_done(const HostFlag &f) {
 // waiting, kv, gpu_util, ttft, tpot) into the six device arrays, which m.running
 // starts (they are contiguous, in that order).
 cudaError_t launch_snapshot(const Model &m, const uint32_t *stage, cudaStream_t s);
-// Fused gather -> MLP -> mask -> argmax for a batch, on nsm SMs.  status: the
+// Fused gather -> MLP -> mask -> argmax for a batch, on nsm SMs.  kernel: 0 the
+// one of small batches, 1 the one of large batches, -1 by the rule.  status: the
 // device status word (bounded waits).  flag (its count and target are filled
 // from `blocks`, a running count of the blocks launched on the counter): the host
 // word to set at the end; *flagged: whether the kernel chosen does.
-cudaError_t launch_route_simt(const Model &m, const Queries &q, int nsm, int32_t *status,
+cudaError_t launch_route_simt(const Model &m, const Queries &q, int nsm, int kernel, int32_t *status,
                               HostFlag flag, uint32_t *blocks, bool *flagged, cudaStream_t s);
 // Small-batch (latency) variant: groups of (query, deployment) pairs with
 // layer 2 split by columns over several blocks, plus quality blocks; scratch

@@ -2283,33 +2283,59 @@ static cudaError_t launch_rows(const Model &m, const Queries &q, int nsm, int32_
     return cudaGetLastError();
 }
 
-// Which of the two batch kernels: k_route_rows once k_route_simt's blocks (64
-// rows; 3 an SM, 2 with more than 128 columns) would take more than one round.
-// Below that the fused blocks' short critical path wins, above it the tile
-// that keeps the FMA pipe busy.  Measured (us, simt / rows, E = 768 where not
-// said): H = 128, D = 12: 24,000 pairs 37.5 / 39.2, 36,000 49.5 / 49.5, 48,012
-// 68.0 / 55.4, 1.2 M 1,330 / 969; H = 128, D = 64: 32,000 62.7 / 53.6; H = 64:
-// 24,000 22.9 / 31.2, 48,000 39.4 / 36.9, 1.2 M 760 / 396; H = 32: 48,000
-// 31.4 / 33.1, 96,000 57.9 / 35.2, 1.2 M 610 / 236; H = 256: 18,000 71.2 /
-// 82.6, 30,000 134 / 103, 240,000 850 / 756.
-// With few deployments a query's quality chains weigh more, and at 65 to 128
-// columns (two deciding warps) they bound k_route_rows: up to 4 deployments it
-// gains nothing there (D = 4, E = 1024: 40,000 pairs 80 / 92, 320,000 434 /
-// 442), up to 7 from about three rounds on (D = 6, E = 1024: 60,000 97 / 102,
-// 120,000 175 / 161).
-// At up to 64 columns the line stays: D = 4, E = 1024 loses only around 80,000
-// pairs (H = 32 85 / 91, H = 64 93 / 98) and gains at 40,000 and from 160,000 on.
-static bool rows_kernel(const Model &m, int Q, int nsm) {
-    const long pairs = (long)Q * m.D, round = 64L * (m.H2 <= 128 ? 3 : 2) * nsm;
-    if (m.H2 > 64 && m.H2 <= 128 && m.D < 8) return m.D > 4 && pairs > 3 * round;
-    return pairs > round;
+// Which of the two batch kernels.  Up to one round of k_route_simt's blocks (64
+// rows; 3 an SM, 2 with more than 128 columns) its short critical path wins.
+// Above, k_route_rows keeps the FMA pipe busier, unless its deciding warps'
+// quality chains (E x M a query, 32 or 16 queries a warp, 16 models a pass) take
+// longer than the tiles (D x H1 x H2 a query): k_route_simt has a warp for them
+// in every block.  Where the chains stay under 0.6 of the tiles and a query has
+// 4 deployments or more, k_route_rows is taken; elsewhere both kernels' times
+// are estimated (us, GB300) from those parts and the smaller wins.  The
+// constants are fitted to 2,861 shapes (D 1 to 64, M 1 to 64, E 8 to 8,192, H1
+// and H2 16 to 256, one round to sixteen) within 9 % and 7 % (rms of the logs),
+// the embeddings' type (bf) to 200 more; over 500 others the choice costs 0.9 %
+// on average against the better kernel, at most a third (32 / 44 us).
+// Measured (us, simt / rows): H = 128, D = 12, E = 768: 1.2 M pairs 1,330 / 969;
+// H = 128, D = M = 64, E = 1,024: 30,000 pairs 100 / 191, 146,000 291 / 234;
+// H = 64, D = 4, M = 2, E = 4,096: 88,000 310 / 323, 233,000 813 / 511; H = 256,
+// D = 12, E = 1,024: 27,000 109 / 102, 97,000 361 / 307.
+static bool rows_kernel(const Model &m, int Q, bool bf, int nsm) {
+    const int D = m.D, M = m.M, W = tile_width(m.H2), per = W == 256 ? 2 : 3;
+    if ((long)Q * D <= 64L * per * nsm) return false;
+    const double hk = (m.H1 + 31) / 32, fma = hk * W / 256;     // 32 x 256 multiply-adds a row
+    const double three = m.NH == 3 ? 1.0 : 0.0;
+    auto up = [](long a, long b) { return (a + b - 1) / b; };
+    // k_route_rows: the deciding warps' and the scoring warps' time
+    const int nq = W <= 64 ? 4 : 2, nw = 16 - nq, rg = W == 256 ? 8 : 16, qbk = D > 32 ? 16 : 32;
+    const long q = up(Q, nsm);
+    const int cols = M < QUAL_MC ? M : QUAL_MC, ng = (cols + 4 * (32 / qbk) - 1) / (4 * (32 / qbk));
+    const double chunk = (bf ? 0.55 : 0.63) + (bf ? 0.2 : 0.15) * (ng == 3 ? 4 : ng) +
+                         (M <= QUAL_MC && M % 4 == 0 ? 0.0 : 0.4);
+    const double dec = up(up(q, qbk), nq) * (up(M, QUAL_MC) * up(m.E, QUAL_KC) * chunk + 5.0);
+    const double group = 3.3 + 0.6 * hk + 2.7 * three +
+                         (W == 256 ? 7.5 : W == 128 ? 7.4 : 6.6) * fma * nw * rg / 192.0;
+    const double score = up(up(q * D, rg), nw) * group;
+    if (D >= 4 && dec < 0.6 * score) return true;
+    const double rows = 7.5 + (dec > score ? dec + 0.4 * score : score + 0.4 * dec);
+    // k_route_simt: waves of `per` blocks an SM, each the longer of its tiles and
+    // its quality chains and half the other
+    const int qb = route_qb(D);
+    const double chains = 1e-3 * m.E * (8.6 + (bf ? 0.55 : 0.9) * qb + 0.32 * M + (qb * M > 32 ? 5.7 : 0.0));
+    const double block = 1.6 + (W >= 128 ? 3.35 : 4.2) * fma + 1.1 * three;
+    auto wave = [&](long n) {
+        const double tile = n * block > 3.2 * hk ? n * block : 3.2 * hk;
+        return tile > chains ? tile + 0.5 * chains : chains + 0.5 * tile;
+    };
+    const long blocks = up(Q, qb), full = blocks / ((long)per * nsm), rest = up(blocks - full * per * nsm, nsm);
+    const double simt = 8.0 + full * wave(per) + (rest ? wave(rest) : 0.0);
+    return rows < simt;
 }
 
-cudaError_t launch_route_simt(const Model &m, const Queries &q, int nsm, int32_t *status,
+cudaError_t launch_route_simt(const Model &m, const Queries &q, int nsm, int kernel, int32_t *status,
                               HostFlag flag, uint32_t *blocks_done, bool *flagged, cudaStream_t s) {
     *flagged = false;
     if (q.Q <= 0) return cudaSuccess;
-    if (rows_kernel(m, q.Q, nsm)) {
+    if (kernel < 0 ? rows_kernel(m, q.Q, q.emb_bf16, nsm) : kernel == 1) {
         switch (tile_width(m.H2)) {
             case 32: return launch_rows<32>(m, q, nsm, status, s);
             case 64: return launch_rows<64>(m, q, nsm, status, s);

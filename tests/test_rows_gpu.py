@@ -4,8 +4,9 @@ and their remainders, K chunks resident and in the ring (H1 above four chunks
 at W = 128, three at W = 256), query blocks of 32 and 16 (D above 32) and
 their remainders, model columns staged as whole rows, padded, and in several
 passes, embedding tails, three heads, bf16 embeddings, unaligned device
-embeddings, and one query more or less than the batch size at which the
-kernel takes over."""
+embeddings (the kernel is asked for by HWR_TEST_BATCH_KERNEL); one query more or
+less than a round of the fused kernel's blocks; and the rule between the two
+kernels, by their times."""
 import numpy as np
 import pytest
 
@@ -32,7 +33,7 @@ def _check(p, got, idx=None):
         assert np.array_equal(np.asarray(g), np.asarray(w).astype(t), equal_nan=True)
 
 
-# (Q, M, G, H1, H2, E, dtype, heads): all above the take-over size
+# (Q, M, G, H1, H2, E, dtype, heads)
 CASES = [
     (7500, 2, 2, 32, 32, 64, "f32", 2),
     (5900, 5, 1, 17, 31, 40, "f32", 3),
@@ -71,7 +72,8 @@ CASES = [
 
 
 @pytest.mark.parametrize("c", CASES, ids=lambda c: "-".join(map(str, c)))
-def test_large_batches_match_the_oracle(c):
+def test_large_batches_match_the_oracle(c, monkeypatch):
+    monkeypatch.setenv("HWR_TEST_BATCH_KERNEL", "1")
     p = _problem(*c)
     r = H.Router(p)
     _check(p, r.route(flags=H.HWR_PATH_SIMT))
@@ -92,8 +94,49 @@ def test_batches_around_the_take_over_size(H2, per):
     r.close()
 
 
-def test_budgets_scores_lambdas_and_unaligned_embeddings():
+# many models and few queries a block, long embeddings with few deployments:
+# the deciding warps' chains bound the kernel of large batches; the others are
+# its own ground
+@pytest.mark.parametrize("Q,M,G,H1,H2,E", [(465, 64, 1, 128, 128, 1024), (930, 32, 1, 32, 32, 2048),
+                                           (9728, 3, 2, 64, 64, 4096), (1915, 20, 1, 64, 50, 3672),
+                                           (8000, 4, 3, 128, 128, 256), (5000, 8, 2, 256, 256, 64)])
+def test_the_rule_takes_the_faster_kernel(Q, M, G, H1, H2, E, monkeypatch):
     import torch
+    p = W.make_problem(Q=1, M=M, G=G, F=M + G + 9, H1=H1, H2=H2, E=E, dtype="f32", lam=0.4, slo=3.0, seed=5)
+    st = torch.cuda.Stream()
+    with torch.cuda.stream(st):
+        il, ol = torch.rand(Q, device="cuda") * 2000 + 16, torch.rand(Q, device="cuda") * 500 + 1
+        emb = torch.randn(Q, E, device="cuda") / E ** 0.5
+        out = [torch.empty(Q, dtype=t, device="cuda") for t in (torch.int32, torch.float32, torch.float32)]
+    st.synchronize()
+    t, got = {}, {}
+    for k in ("0", "1", None):
+        if k is None:
+            monkeypatch.delenv("HWR_TEST_BATCH_KERNEL")
+        else:
+            monkeypatch.setenv("HWR_TEST_BATCH_KERNEL", k)
+        r = H.Router(p, stream=st.cuda_stream)
+        best = 1e9
+        for _ in range(6):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record(st)
+            for _ in range(5):
+                r.route_device(il, ol, emb, *out, slo=3.0, lam=0.4, flags=H.HWR_ASYNC)
+            b.record(st)
+            b.synchronize()
+            best = min(best, a.elapsed_time(b))
+        r.synchronize()
+        t[k], got[k] = best, [o.cpu().numpy() for o in out]
+        r.close()
+    for k in ("1", None):
+        for x, y in zip(got[k], got["0"]):
+            assert np.array_equal(x, y, equal_nan=True)
+    assert t[None] < 1.35 * min(t["0"], t["1"]), t
+
+
+def test_budgets_scores_lambdas_and_unaligned_embeddings(monkeypatch):
+    import torch
+    monkeypatch.setenv("HWR_TEST_BATCH_KERNEL", "1")
     p = _problem(2500, 4, 3, 128, 128, 64)
     st = torch.cuda.Stream()
     r = H.Router(p, stream=st.cuda_stream)
