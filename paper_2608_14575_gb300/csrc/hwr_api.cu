@@ -77,6 +77,7 @@ struct hwr_ctx {
     int test_stall = 0;          // HWR_TEST_STALL: tensor-path producers never signal
     int tc_min_pairs = TC_MIN_PAIRS, pairs_max = -1;   // -1: by the context's paths
     int batch_kernel = -1;       // HWR_TEST_BATCH_KERNEL: the fp32 batch kernel (launch_route_simt)
+    int seq_chunk = 0;           // HWR_TEST_SEQ_CHUNK: queries per chunk of the SIMT sequential table
     int device = -1;             // the CUDA device current at hwr_create
     long poll_us = 1000000;      // limit of the host's polls (HWR_TEST_POLL_US)
     bool async_pending = false;  // an HWR_ASYNC call may still have work queued
@@ -641,6 +642,7 @@ extern "C" hwr_status hwr_create(const hwr_deployment_table *table, const hwr_pr
         c->ats = pageable == 1 && !(h && atoi(h) != 0);
     }
     if (const char *h = getenv("HWR_TEST_STALL")) c->test_stall = atoi(h) != 0;
+    if (const char *h = getenv("HWR_TEST_SEQ_CHUNK")) c->seq_chunk = atoi(h);
     if (const char *h = getenv("HWR_TEST_BATCH_KERNEL")) c->batch_kernel = atoi(h) == 1 ? 1 : 0;
     if (const char *h = getenv("HWR_TC_MIN_PAIRS")) c->tc_min_pairs = atoi(h) > 1 ? atoi(h) : 1;
     if (const char *h = getenv("HWR_PAIRS_MAX_PAIRS"))
@@ -765,7 +767,8 @@ static hwr_status run_kernels(hwr_ctx *c, const Queries &q, uint32_t flags, bool
         // rows that do not fit its shared memory from L2.
         const int nchunks = (q.Q + SEQ_MAX_CHUNK - 1) / SEQ_MAX_CHUNK;
         const int Qs = tcs ? (q.Q + nchunks - 1) / nchunks
-                           : seq_pick_chunk(m, q.Q, c->seq_qs, c->seq_slots);
+                       : c->seq_chunk > 0 ? (c->seq_chunk < c->seq_qs ? c->seq_chunk : c->seq_qs)
+                                          : seq_pick_chunk(m, q.Q, c->seq_qs, c->seq_slots);
         if (tcs) {
             const size_t Dv = (size_t)c->D * (Qs + 1);
             TRY(grow(c, &c->prebf, &c->prebf_cap, Dv * c->H1));

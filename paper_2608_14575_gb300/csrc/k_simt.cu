@@ -2438,24 +2438,35 @@ static SeqGrid seq_grid(const Model &m, int Qs, int slots) {
 
 // Queries per chunk of a sequential call of Q.  A chunk costs a fixed part (its
 // launches, the tables' serial parts, the walk and its copy) and its table's
-// rounds of blocks of rpb rows; the table grows with the square of a chunk, so
-// wide clusters take shorter chunks.  Both parts grow with H1; the constants
-// fit chunks of 8 to 64 queries measured on GB300 (us: H = 64, D = 32: 9.8 and
-// 0.14 a row; H = 128, D = 12: 13.5 and 0.38; H = 256, D = 32: 20 and 0.85;
-// shorter blocks than 24 rows wait on latencies and take as long).
+// rounds of blocks of rpb rows, the last one 0.6 of a round and the rest in
+// proportion; the table grows with the square of a chunk, so wide clusters take
+// shorter chunks.  Both parts grow with H1 and with the width W of the table's
+// tile, here by their geometric mean.  Blocks below 32 rows wait on latencies and
+// take as long; at W = 256 those above 60 gain as much by hiding them.  The
+// constants fit chunks of 8 to 64 queries of 31 shapes measured on GB300, H1 and
+// H2 apart in half of them (us: H = 64, D = 32: 9.8 and 0.17 a row; H = 128, D =
+// 12: 13.2 and 0.38; H = 256, D = 32: 20 and 0.80): over them the choice is 0.2 %
+// from the best chunk on average, 6 % at most; of 450 other shapes five are over
+// 3 % slower than in the largest chunks (at most 11 %, 46 / 51 us).
 // 1,000 requests in the largest chunks that the chain takes / in the ones
-// chosen here (us): D = 12, H = 128 548 / 526; D = 32, H = 64 494 / 456;
-// D = 32, H = 256 2,689 / 1,737; D = 64, H = 256 4,432 / 3,032.
+// chosen here (us): D = 12, H = 128 541 / 511; D = 32, H = 64 479 / 458; D = 32,
+// H = 256 2,674 / 1,726; D = 64, H = 256 4,433 / 2,719; D = 32, H1 = 32, H2 = 256
+// 686 / 583; D = 32, H1 = 256, H2 = 32 974 / 940.
 int seq_pick_chunk(const Model &m, int Q, int limit, int slots) {
-    const double fixed_us = 6.4 + 0.053 * m.H1;
-    const double row_us = m.H1 > 21 ? 0.0033 * m.H1 - 0.04 : 0.03;
+    const int W = tile_width(m.H2), most = W == 256 ? 60 : TILE_ROWS;
+    const double h = sqrt((double)m.H1 * W);
+    const double fixed_us = 6.4 + 0.053 * h;
+    const double row_us = h > 21 ? 0.0033 * h - 0.04 : 0.03;
     int best = limit;
     double best_cost = 1e300;
     for (int n = (Q + limit - 1) / limit;; ++n) {
         const int Qs = (Q + n - 1) / n;
         const SeqGrid g = seq_grid(m, Qs, slots);
-        const double rounds = g.blocks > slots ? (double)g.blocks / slots : 1.0;
-        const double cost = ((Q + Qs - 1) / Qs) * (fixed_us + row_us * (g.rpb > 24 ? g.rpb : 24) * rounds);
+        const double part = (double)((g.blocks - g.nb_qual) % slots) / slots;
+        double rounds = (g.blocks - g.nb_qual) / slots + (part > 0.0 ? 0.6 + 0.4 * part : 0.0);
+        if (rounds < 1.0) rounds = 1.0;
+        const int rows = g.rpb < 32 ? 32 : g.rpb > most ? most : g.rpb;
+        const double cost = ((Q + Qs - 1) / Qs) * (fixed_us + row_us * rows * rounds);
         if (cost < best_cost) {
             best_cost = cost;
             best = Qs;
