@@ -77,6 +77,7 @@ struct hwr_ctx {
     int test_stall = 0;          // HWR_TEST_STALL: tensor-path producers never signal
     int tc_min_pairs = TC_MIN_PAIRS, pairs_max = -1;   // -1: by the context's paths
     int batch_kernel = -1;       // HWR_TEST_BATCH_KERNEL: the fp32 batch kernel (launch_route_simt)
+    bool poll_only = false;      // HWR_TEST_POLL_ONLY: a waited device call must end by its host word
     int seq_chunk = 0;           // HWR_TEST_SEQ_CHUNK: queries per chunk of the SIMT sequential table
     int device = -1;             // the CUDA device current at hwr_create
     long poll_us = 1000000;      // limit of the host's polls (HWR_TEST_POLL_US)
@@ -642,6 +643,7 @@ extern "C" hwr_status hwr_create(const hwr_deployment_table *table, const hwr_pr
         c->ats = pageable == 1 && !(h && atoi(h) != 0);
     }
     if (const char *h = getenv("HWR_TEST_STALL")) c->test_stall = atoi(h) != 0;
+    if (const char *h = getenv("HWR_TEST_POLL_ONLY")) c->poll_only = atoi(h) != 0;
     if (const char *h = getenv("HWR_TEST_SEQ_CHUNK")) c->seq_chunk = atoi(h);
     if (const char *h = getenv("HWR_TEST_BATCH_KERNEL")) c->batch_kernel = atoi(h) == 1 ? 1 : 0;
     if (const char *h = getenv("HWR_TC_MIN_PAIRS")) c->tc_min_pairs = atoi(h) > 1 ? atoi(h) : 1;
@@ -1292,9 +1294,12 @@ static hwr_status route_impl(hwr_ctx *c, int32_t Q, const float *in_len, const f
         c->async_pending = true;
         return HWR_OK;
     }
-    if (!synced && !(c->flagged && wait_flag(c->flag_h, c->flag_seq,
-                                             c->poll_us < FLAG_POLL_US ? c->poll_us : FLAG_POLL_US)))
-        CK(c, cudaStreamSynchronize(c->stream), "synchronize");
+    if (!synced) {
+        const long limit = c->poll_only || c->poll_us < FLAG_POLL_US ? c->poll_us : FLAG_POLL_US;
+        const bool seen = c->flagged && wait_flag(c->flag_h, c->flag_seq, limit);
+        if (!seen) CK(c, cudaStreamSynchronize(c->stream), "synchronize");
+        if (!seen && c->poll_only) return fail(c, HWR_ERR_TIMEOUT, "no host word ended the call (test hook)");
+    }
     // this call's work is complete, and with it every earlier kernel
     c->async_pending = false;
     c->snap_busy = false;

@@ -2,7 +2,9 @@
 sets.  Outputs copied on another stream right after the return, without any
 synchronisation, must be complete; inputs may be overwritten from another
 stream; the synchronising fallback (limit 0) and calls behind queued work give
-the same results.  Fused fp32 kernel and tensor path, split and whole tiles."""
+the same results.  Fused fp32 kernel and tensor path, split and whole tiles.
+That the word does end such calls, over many grids and both paths in turn, is
+asked for by HWR_TEST_POLL_ONLY, under which a call that falls back fails."""
 import numpy as np
 import pytest
 import torch
@@ -50,4 +52,27 @@ def test_outputs_are_complete_at_the_return(monkeypatch, dtype, M, G, H1, Q, pol
     for i in range(20):
         for k, w in zip(kept[i], want[i % 2]):
             assert np.array_equal(k.cpu().numpy(), w, equal_nan=True), i
+    r.close()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_the_host_word_ends_waited_calls(monkeypatch, dtype):
+    monkeypatch.setenv("HWR_TEST_POLL_ONLY", "1")
+    p = W.make_problem(Q=3000, M=4, G=2, F=18, H1=64, H2=64, E=64, dtype=dtype, lam=0.4, slo=2.0, seed=6,
+                       bias_std=0.05)
+    st = torch.cuda.Stream()
+    r = H.Router(p, stream=st.cuda_stream)
+    ins = [torch.from_numpy(p[k].view(np.int16) if p[k].dtype == np.uint16 else p[k]).cuda()
+           for k in ("in_len", "out_len", "emb")]
+    out = [torch.empty(3000, dtype=t, device="cuda") for t in (torch.int32, torch.float32, torch.float32)]
+    torch.cuda.synchronize()
+    for i, Q in enumerate((3000, 97, 1024, 2999, 100, 513, 1500, 3000) * 4):
+        path = H.HWR_PATH_TENSOR if dtype == "bf16" and i % 3 else H.HWR_PATH_SIMT
+        r.route_device(*(t[:Q] for t in ins), *(o[:Q] for o in out), slo=p["slo"], lam=p["lam"], flags=path)
+    r.close()
+    # the fallback shows: nothing polls here
+    monkeypatch.setenv("HWR_TEST_POLL_US", "0")
+    r = H.Router(p, stream=st.cuda_stream)
+    with pytest.raises(H.HwrError, match="host word"):
+        r.route_device(*ins, *out, slo=p["slo"], lam=p["lam"], flags=path)
     r.close()
