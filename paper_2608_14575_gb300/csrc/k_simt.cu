@@ -1366,13 +1366,13 @@ k_seq_chain(Model m, Queries q, int Qs, int Ns, const float *ctab, float *aux, c
         auto steps = [&](int lo, int hi, uint32_t &rec0, uint32_t &rec1) {
 #pragma unroll 2
             for (int i = lo; i < hi; ++i) {
-                const bool more = i + 1 < Qs;
-                const float b = slo[more ? i + 1 : i];
-                qn0 += more ? M : 0;
+                const bool next = i + 1 < Qs;
+                const float b = slo[next ? i + 1 : i];
+                qn0 += next ? M : 0;
                 const float q0 = *qn0, x0s = at(a0), x0p = at(a0p);
                 float q1 = 0.f, x1s = 0.f, x1p = 0.f;
                 if (HI) {
-                    qn1 += more ? M : 0;
+                    qn1 += next ? M : 0;
                     q1 = *qn1;
                     x1s = at(a1);
                     x1p = at(a1p);
@@ -1406,10 +1406,10 @@ k_seq_chain(Model m, Queries q, int Qs, int Ns, const float *ctab, float *aux, c
             start();
 #pragma unroll 1
             for (int i = 0; i < Qs; ++i) {
-                const bool more = i + 1 < Qs;
-                const float b = slo[more ? i + 1 : i], bi = slo[i];
-                qn0 += more ? M : 0;
-                qn1 += HI && more ? M : 0;
+                const bool next = i + 1 < Qs;
+                const float b = slo[next ? i + 1 : i], bi = slo[i];
+                qn0 += next ? M : 0;
+                qn1 += HI && next ? M : 0;
                 const float x0s = at(a0), x0p = at(a0p), x1s = HI ? at(a1) : 0.f, x1p = HI ? at(a1p) : 0.f;
                 // the classes in turn: feasible with a defined utility (-inf among
                 // them), any defined cost, none

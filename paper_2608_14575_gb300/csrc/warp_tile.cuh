@@ -1,7 +1,7 @@
-// The fp32 tile of the SIMT kernels: one warp scores RG rows, each a (query,
-// deployment) pair or a sequential-table entry, from a deployment prefix of
-// layer 1 and two query features to the cost, in canonical order (every dot
-// product bias first, k ascending, one fused rounding per step).
+// The fp32 tile of the large-batch kernel: one warp scores RG rows, each a (query,
+// deployment) pair, from a deployment prefix of layer 1 and two query features to
+// the cost, in canonical order (every dot product bias first, k ascending, one
+// fused rounding per step).
 //
 // What bounds it is the FMA pipe (128 a cycle and SM), so the layout keeps
 // everything else off its way:
@@ -30,11 +30,11 @@ namespace hwr {
 
 constexpr int TILE_KC = 32;
 
-// Lane tile of a group of RG rows with W columns: LC columns and LR rows a
-// lane, NSET sets of rows.
+// Lane tile of a group of RG rows with W columns (8 rows at W = 256, else 16): LC
+// columns and LR rows a lane, NSET sets of rows.
 template <int W, int RG>
 struct Tile {
-    static constexpr int LC = W == 256 ? 8 : W * RG >= 2048 ? 8 : W * RG >= 1024 ? 4 : W * RG >= 512 ? 2 : 1;
+    static constexpr int LC = W >= 128 ? 8 : W == 64 ? 4 : 2;
     static constexpr int NSET = 32 * LC / W, LR = RG / NSET;
     static constexpr int LD = RG + 4;                    // layer-1 chunk [TILE_KC][LD], k-major:
                                                          // a lane's 16-byte stores of its k fall in
@@ -42,7 +42,7 @@ struct Tile {
     static constexpr int PIECE = W < 64 ? 32 : 64;       // layer-2 columns the head chains read at a time
     static constexpr int PLD = PIECE + 4;                // their row stride: odd in 16-byte units
     static constexpr int BUF = TILE_KC * LD > RG * PLD ? TILE_KC * LD : RG * PLD;
-    static_assert(LR >= 4 && LR % 4 == 0 && NSET >= 1 && (RG == 8 || RG == 16), "lane tile");
+    static_assert(LR == 8 && NSET >= 1 && RG == (W == 256 ? 8 : 16), "lane tile");
 };
 
 // One row as the tile reads it: standardised query slots, offset of the
@@ -131,7 +131,7 @@ __device__ __forceinline__ bool w2_skip(const W2Feed &f, uint32_t n0) {
 // The block's weights that every row uses, in shared memory.
 struct TileWeights {
     const float *w1q;   // [2][H1]: W1's query columns
-    const float *b2;    // [32 CPT], zero past H2
+    const float *b2;    // [W], zero past H2
     const float *w3;    // [NH][H2p]
     const float *b3;    // [NH]
 };
@@ -178,12 +178,10 @@ __device__ __forceinline__ void tile_step(uint32_t ar, uint32_t wr, float2 (&acc
             b[4 * v + 1] = t.y;
             b[4 * v + 2] = t.z;
             b[4 * v + 3] = t.w;
-        } else if constexpr (VW == 2) {
+        } else {
             const float2 t = lds2(wr);
             b[0] = t.x;
             b[1] = t.y;
-        } else {
-            b[0] = lds1(wr);
         }
     }
     // each lane of the packed FMA rounds once, as __fmaf_rn
