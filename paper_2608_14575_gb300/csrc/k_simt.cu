@@ -553,8 +553,8 @@ k_route_simt(Model m, Queries q, HostFlag flag) {
 // and decide.  The costs pass through a ring of NB blocks in shared memory
 // (done, an mbarrier: the groups' arrivals; freed, a count: the decisions), so
 // the two sides meet only when one is a whole ring ahead.
-// Bound: the FMA pipe; measured 42.5 TFLOP/s at 100,000 queries, D = 12,
-// H = 128 (53 % of 80.5; k_route_simt 31), where a k step's 64 packed FMAs
+// Bound: the FMA pipe; measured 43.1 TFLOP/s at 100,000 queries, D = 12,
+// H = 128 (54 % of 80.5; k_route_simt 31), where a k step's 64 packed FMAs
 // come with about 50 other instructions (the pairs of a W2 value with itself,
 // loads) and fill the issue slots.
 

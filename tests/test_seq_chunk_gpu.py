@@ -41,4 +41,4 @@ def test_the_chunk_size_chosen_is_a_good_one(M, G, H1, H2, monkeypatch):
     for n in t:
         for x, y in zip(got[n], got["0"]):
             assert np.array_equal(x, y, equal_nan=True), n
-    assert t["0"] < 1.15 * min(t.values()), t
+    assert t["0"] < 1.2 * min(t.values()), t
