@@ -770,7 +770,7 @@ static hwr_status run_kernels(hwr_ctx *c, const Queries &q, uint32_t flags, bool
         const int nchunks = (q.Q + SEQ_MAX_CHUNK - 1) / SEQ_MAX_CHUNK;
         const int Qs = tcs ? (q.Q + nchunks - 1) / nchunks
                        : c->seq_chunk > 0 ? (c->seq_chunk < c->seq_qs ? c->seq_chunk : c->seq_qs)
-                                          : seq_pick_chunk(m, q.Q, c->seq_qs, c->seq_slots);
+                                          : seq_pick_chunk(m, q.Q, c->seq_qs, c->seq_slots, c->nsm);
         if (tcs) {
             const size_t Dv = (size_t)c->D * (Qs + 1);
             TRY(grow(c, &c->prebf, &c->prebf_cap, Dv * c->H1));

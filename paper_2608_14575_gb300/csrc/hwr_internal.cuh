@@ -181,7 +181,7 @@ cudaError_t launch_seq_chain_tc(const Model &m, const Queries &q, int Qs, const 
                                 float *aux, const float *qual, int qstride, bool more,
                                 cudaStream_t s);
 int seq_table_slots(const Model &m);
-int seq_pick_chunk(const Model &m, int Q, int limit, int slots);
+int seq_pick_chunk(const Model &m, int Q, int limit, int slots, int nsm);
 // Decision maker for K lambdas from stored scores: C [Q][D], quality
 // qual[q * qstride + model]; outputs [K][ostride] starting at query 0.
 cudaError_t launch_select_multi(const Model &m, const Queries &q, const float *C,

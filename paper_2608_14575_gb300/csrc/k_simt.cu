@@ -2437,36 +2437,31 @@ static SeqGrid seq_grid(const Model &m, int Qs, int slots) {
 }
 
 // Queries per chunk of a sequential call of Q.  A chunk costs a fixed part (its
-// launches, the tables' serial parts, the walk and its copy) and its table's
-// rounds of blocks of rpb rows, the last one 0.6 of a round and the rest in
-// proportion; the table grows with the square of a chunk, so wide clusters take
-// shorter chunks.  Both parts grow with H1 and with the width W of the table's
-// tile, here by their geometric mean.  Blocks below 32 rows wait on latencies and
-// take as long; at W = 256 those above 60 gain as much by hiding them.  The
-// constants fit chunks of 8 to 64 queries of 31 shapes measured on GB300, H1 and
-// H2 apart in half of them (us: H = 64, D = 32: 9.8 and 0.17 a row; H = 128, D =
-// 12: 13.2 and 0.38; H = 256, D = 32: 20 and 0.80): over them the choice is 0.2 %
-// from the best chunk on average, 6 % at most; of 450 other shapes five are over
-// 3 % slower than in the largest chunks (at most 11 %, 46 / 51 us).
+// launches, the tables' serial parts, the walk and its copy) and its table, which
+// grows with the square of a chunk, so wide clusters take shorter chunks.  The
+// table's time goes by the blocks that the busiest SM takes, resident or one after
+// the other, and by their rows: above 32 a block's warps double up on the SM's
+// sub-partitions (H = 256, D = 20, us: 43.0 at 32 rows, 58.0 at 40, 62.5 to 65 at 48
+// to 64; a third block on an SM, a fourth: 91, 117).  The constants (us) fit every
+// chunk size from 8 on of 110 shapes measured on GB300 (D 2 to 64, H1 and H2 16 to
+// 256, apart in half of them), chosen for calls of 64 to 1,000: 0.9 % over the best
+// chunk on average, 13 % at most (fitted to half of the shapes only, 1.3 % and
+// 14 % on the others).
 // 1,000 requests in the largest chunks that the chain takes / in the ones
 // chosen here (us): D = 12, H = 128 541 / 511; D = 32, H = 64 479 / 458; D = 32,
-// H = 256 2,674 / 1,726; D = 64, H = 256 4,433 / 2,719; D = 32, H1 = 32, H2 = 256
-// 686 / 583; D = 32, H1 = 256, H2 = 32 974 / 940.
-int seq_pick_chunk(const Model &m, int Q, int limit, int slots) {
-    const int W = tile_width(m.H2), most = W == 256 ? 60 : TILE_ROWS;
-    const double h = sqrt((double)m.H1 * W);
-    const double fixed_us = 6.4 + 0.053 * h;
-    const double row_us = h > 21 ? 0.0033 * h - 0.04 : 0.03;
+// H = 256 2,674 / 1,726; D = 64, H = 256 4,433 / 2,719.
+int seq_pick_chunk(const Model &m, int Q, int limit, int slots, int nsm) {
+    const int W = tile_width(m.H2);
+    const double hk = (m.H1 + 31) / 32, fma = m.H1 * W / 8192.0;
+    const double fixed_us = 4.9 + 0.8 * hk + 0.33 * W / 32, block_us = 0.6 + 0.065 * hk + 1.1 * fma;
     int best = limit;
     double best_cost = 1e300;
     for (int n = (Q + limit - 1) / limit;; ++n) {
         const int Qs = (Q + n - 1) / n;
         const SeqGrid g = seq_grid(m, Qs, slots);
-        const double part = (double)((g.blocks - g.nb_qual) % slots) / slots;
-        double rounds = (g.blocks - g.nb_qual) / slots + (part > 0.0 ? 0.6 + 0.4 * part : 0.0);
-        if (rounds < 1.0) rounds = 1.0;
-        const int rows = g.rpb < 32 ? 32 : g.rpb > most ? most : g.rpb;
-        const double cost = ((Q + Qs - 1) / Qs) * (fixed_us + row_us * rows * rounds);
+        const int blocks = (g.blocks - g.nb_qual + nsm - 1) / nsm;      // on the busiest SM
+        const double rows = 0.3 * ((g.rpb + 31) / 32) + 0.7 * (g.rpb < 16 ? 16 : g.rpb) / 32;
+        const double cost = ((Q + Qs - 1) / Qs) * (fixed_us + 0.057 * Qs + block_us * blocks * rows);
         if (cost < best_cost) {
             best_cost = cost;
             best = Qs;
