@@ -2291,11 +2291,11 @@ static cudaError_t launch_rows(const Model &m, const Queries &q, int nsm, int32_
 // in every block.  Where the chains stay under 0.6 of the tiles and a query has
 // 4 deployments or more, k_route_rows is taken; elsewhere both kernels' times
 // are estimated (us, GB300) from those parts and the smaller wins.  The
-// constants are fitted to 2,861 shapes (D 1 to 64, M 1 to 64, E 8 to 8,192, H1
-// and H2 16 to 256, one round to sixteen) within 9 % and 7 % (rms of the logs),
-// the embeddings' type (bf) to 200 more; over 500 others the choice costs 0.9 %
-// on average against the better kernel, at most a third (32 / 44 us).
-// Measured (us, simt / rows): H = 128, D = 12, E = 768: 1.2 M pairs 1,330 / 969;
+// constants were chosen on 4,861 measured shapes (D 1 to 64, M 1 to 64, E 8 to
+// 8,192, H1 and H2 1 to 256, one round to sixteen, fp32 and bf16 embeddings) so
+// that the choice costs least: 0.5 % over the better kernel on average on them,
+// 0.9 % on 900 others (the worst: 17 / 27 us at H1 = 1, D = 64, M = 4).
+// Measured (us, simt / rows): H = 128, D = 12, E = 768: 1.2 M pairs 1,330 / 954;
 // H = 128, D = M = 64, E = 1,024: 30,000 pairs 100 / 191, 146,000 291 / 234;
 // H = 64, D = 4, M = 2, E = 4,096: 88,000 310 / 323, 233,000 813 / 511; H = 256,
 // D = 12, E = 1,024: 27,000 109 / 102, 97,000 361 / 307.
@@ -2309,25 +2309,25 @@ static bool rows_kernel(const Model &m, int Q, bool bf, int nsm) {
     const int nq = W <= 64 ? 4 : 2, nw = 16 - nq, rg = W == 256 ? 8 : 16, qbk = D > 32 ? 16 : 32;
     const long q = up(Q, nsm);
     const int cols = M < QUAL_MC ? M : QUAL_MC, ng = (cols + 4 * (32 / qbk) - 1) / (4 * (32 / qbk));
-    const double chunk = (bf ? 0.55 : 0.63) + (bf ? 0.2 : 0.15) * (ng == 3 ? 4 : ng) +
-                         (M <= QUAL_MC && M % 4 == 0 ? 0.0 : 0.4);
-    const double dec = up(up(q, qbk), nq) * (up(M, QUAL_MC) * up(m.E, QUAL_KC) * chunk + 5.0);
-    const double group = 3.3 + 0.6 * hk + 2.7 * three +
-                         (W == 256 ? 7.5 : W == 128 ? 7.4 : 6.6) * fma * nw * rg / 192.0;
+    const double chunk = 0.57 + (bf ? 0.19 : 0.11) * (ng == 3 ? 4 : ng) +
+                         (M <= QUAL_MC && M % 4 == 0 ? 0.0 : 0.51);
+    const double dec = up(up(q, qbk), nq) * (up(M, QUAL_MC) * up(m.E, QUAL_KC) * chunk + 3.22);
+    const double group = 3.31 + 0.62 * hk + 3.22 * three +
+                         (W == 256 ? 7.67 : W == 128 ? 10.59 : 5.88) * fma * nw * rg / 192.0;
     const double score = up(up(q * D, rg), nw) * group;
     if (D >= 4 && dec < 0.6 * score) return true;
-    const double rows = 7.5 + (dec > score ? dec + 0.4 * score : score + 0.4 * dec);
+    const double rows = 8.95 + (dec > score ? dec + 0.47 * score : score + 0.47 * dec);
     // k_route_simt: waves of `per` blocks an SM, each the longer of its tiles and
-    // its quality chains and half the other
+    // its quality chains and a part of the other
     const int qb = route_qb(D);
-    const double chains = 1e-3 * m.E * (8.6 + (bf ? 0.55 : 0.9) * qb + 0.32 * M + (qb * M > 32 ? 5.7 : 0.0));
-    const double block = 1.6 + (W >= 128 ? 3.35 : 4.2) * fma + 1.1 * three;
+    const double chains = 1e-3 * m.E * (9.36 + (bf ? 0.58 : 0.83) * qb + 0.35 * M + (qb * M > 32 ? 5.5 : 0.0));
+    const double block = 1.44 + (W >= 128 ? 3.53 : 5.6) * fma + 1.44 * three;
     auto wave = [&](long n) {
-        const double tile = n * block > 3.2 * hk ? n * block : 3.2 * hk;
-        return tile > chains ? tile + 0.5 * chains : chains + 0.5 * tile;
+        const double tile = n * block > 3.24 * hk ? n * block : 3.24 * hk;
+        return 0.04 * qb + (tile > chains ? tile + 0.59 * chains : chains + 0.59 * tile);
     };
     const long blocks = up(Q, qb), full = blocks / ((long)per * nsm), rest = up(blocks - full * per * nsm, nsm);
-    const double simt = 8.0 + full * wave(per) + (rest ? wave(rest) : 0.0);
+    const double simt = 8.1 + full * wave(per) + (rest ? wave(rest) : 0.0);
     return rows < simt;
 }
 
