@@ -2449,7 +2449,7 @@ static SeqGrid seq_grid(const Model &m, int Qs, int slots) {
 // 14 % on the others).
 // 1,000 requests in the largest chunks that the chain takes / in the ones
 // chosen here (us): D = 12, H = 128 541 / 511; D = 32, H = 64 479 / 458; D = 32,
-// H = 256 2,674 / 1,726; D = 64, H = 256 4,433 / 2,719.
+// H = 256 2,674 / 1,726; D = 64, H = 256 4,433 / 2,786.
 int seq_pick_chunk(const Model &m, int Q, int limit, int slots, int nsm) {
     const int W = tile_width(m.H2);
     const double hk = (m.H1 + 31) / 32, fma = m.H1 * W / 8192.0;
