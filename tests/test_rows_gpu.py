@@ -131,7 +131,9 @@ def test_the_rule_takes_the_faster_kernel(Q, M, G, H1, H2, E, monkeypatch):
     for k in ("1", None):
         for x, y in zip(got[k], got["0"]):
             assert np.array_equal(x, y, equal_nan=True)
-    assert t[None] < 1.35 * min(t["0"], t["1"]), t
+    # (the rule by pairs and widths alone took 1.75 to 1.9 times the better one in the
+    # shapes of many models)
+    assert t[None] < 1.45 * min(t["0"], t["1"]), t
 
 
 def test_budgets_scores_lambdas_and_unaligned_embeddings(monkeypatch):

@@ -41,4 +41,5 @@ def test_the_chunk_size_chosen_is_a_good_one(M, G, H1, H2, monkeypatch):
     for n in t:
         for x, y in zip(got[n], got["0"]):
             assert np.array_equal(x, y, equal_nan=True), n
-    assert t["0"] < 1.2 * min(t.values()), t
+    # (by H1 alone 1.3 times the best of them at 64 x 256 and 32 x 256)
+    assert t["0"] < 1.22 * min(t.values()), t
